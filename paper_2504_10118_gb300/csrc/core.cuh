@@ -27,6 +27,7 @@ constexpr int kApplyUnroll = 4;      // increments in flight per thread in the u
 #include "fft_lines.cuh"
 #include "update.cuh"
 #include "window_kernel.cuh"
+#include "window_split.cuh"
 
 // the window sides with a window kernel
 #define MAGPIE_WINDOW_SIZES(X) X(8) X(16) X(32) X(64) X(128) X(256)
@@ -84,5 +85,13 @@ cudaError_t window_launch_persistent(const PersistArgs& P, int clusters, int max
 // the clusters of the persistent step kernel that fit on the GPU at once.
 template <int MS>
 int window_persistent_capacity(int max_count, int minb);
+// the split form of a minibatch step's window phase (window_split.cuh, sides
+// of 64 and more), its increments stored or added with float atomics; early:
+// the indices are final before the stream's previous kernel ends
+template <int MS>
+cudaError_t split_launch(bool atomic, bool early, const StepArgs& a, int windows, cudaStream_t st);
+// and over the windows of several problems
+template <int MS>
+cudaError_t split_launch_batched(const StepArgs* table, const int2* map, int windows, cudaStream_t st);
 
 }  // namespace magpie_impl

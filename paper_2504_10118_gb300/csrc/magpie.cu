@@ -61,18 +61,21 @@ constexpr int kVersion = 10300;  // 1.3.0
 // kernel that ends the step may run: block (0, 0) zeroes them for the next
 // step (whose exit kernel waits for this grid to complete).
 __device__ __forceinline__ void clear_handoff(const ApplyArgs& P) {
-  if (P.hand && blockIdx.x == 0 && blockIdx.y == 0)
+  if (P.hand && blockIdx.x == 0)
     for (int i = threadIdx.x; i < P.nhand; i += blockDim.x) P.hand[i] = 0;
 }
 
-// One problem: a 2-D grid of tiles.
+// One problem: a block per tile and one for the partial sums.
 // Launched as a programmatic dependent of the window kernel (its blocks, let
 // in early, would slow the next window kernel: 0.328 against 0.319 ms per
 // sweep, so it does not trigger its dependents).
+template <int TW, int TH>
 __global__ void __launch_bounds__(256) apply_kernel(ApplyArgs P) {
-  grid_dep_wait();
-  clear_handoff(P);
-  apply_body<kApplyTile, kApplyTile>(P, blockIdx.x, blockIdx.y);
+  if (P.hand) {
+    grid_dep_wait();
+    clear_handoff(P);
+  }
+  apply_body<TW, TH>(P, blockIdx.x % P.tiles_x, blockIdx.x / P.tiles_x);
 }
 
 // The precision form's update: the same ordered sum, each window's
@@ -80,7 +83,7 @@ __global__ void __launch_bounds__(256) apply_kernel(ApplyArgs P) {
 __global__ void __launch_bounds__(256) apply_tail_kernel(ApplyArgs P) {
   grid_dep_wait();
   clear_handoff(P);
-  apply_body<kApplyTile, kApplyTile, 256, true>(P, blockIdx.x, blockIdx.y);
+  apply_body<16, 16, 256, true>(P, blockIdx.x % P.tiles_x, blockIdx.x / P.tiles_x);
 }
 
 // Several problems in one launch (1-D grid): problem i owns blocks
@@ -469,15 +472,30 @@ ApplyArgs apply_args(float2* z, int n_rows, int n_cols, const int2* corners, con
   return P;
 }
 
-int apply_tiles(const ApplyArgs& P) { return P.tiles_x * P.tiles_y; }
+// blocks of one update: its tiles and the block of the partial sums
+int apply_tiles(const ApplyArgs& P) { return P.tiles_x * P.tiles_y + 1; }
+
+// The update of one problem on its own, in 32 x 32 tiles (four pixels per
+// thread share the window list and its tests) once those are 400 or more, else
+// in 16 x 16 tiles, which keep small objects from leaving SMs idle: step of 64
+// windows with m = 128 (us, 16 x 16 / 32 x 32 tiles): 19.8 / 21.7 at n = 512,
+// 22.6 / 22.1 at 640, 26.1 / 22.6 at 1024; m = 256: 62.6 / 68.0 at n = 600,
+// 63.5 / 62.5 at 768.  The precision form's tail does as well with either.
+cudaError_t launch_apply_args(ApplyArgs P, cudaStream_t st) {
+  const long long big = (long long)((P.n_cols + 31) / 32) * ((P.n_rows + 31) / 32);
+  const ApplyShape s = kApplyShapes[big >= 400 ? 2 : 0];
+  P.tiles_x = (P.n_cols + s.tw - 1) / s.tw;
+  P.tiles_y = (P.n_rows + s.th - 1) / s.th;
+  return launch_ex(big >= 400 ? apply_kernel<32, 32> : apply_kernel<16, 16>, dim3((unsigned)apply_tiles(P)), dim3(256),
+                   sizeof(ApplyEntry) * P.count, st, 1, true, P);
+}
 
 cudaError_t launch_apply(float2* z, int n_rows, int n_cols, const int2* corners, const int32_t* idx, int count,
                          int n_pos, const float2* contrib, const float* w0, int MS, const double* part,
                          double* phi_pos, double* gn_pos, cudaStream_t st, int slots = 0) {
   const ApplyArgs P =
       apply_args(z, n_rows, n_cols, corners, idx, count, n_pos, contrib, w0, MS, part, phi_pos, gn_pos, slots);
-  const dim3 tiles(P.tiles_x, (n_rows + kApplyTile - 1) / kApplyTile);
-  return launch_ex(apply_kernel, tiles, dim3(256), (sizeof(int2) + sizeof(int)) * count, st, 1, true, P);
+  return launch_apply_args(P, st);
 }
 
 template <int MODE>
@@ -506,6 +524,24 @@ cudaError_t launch_window_batched_m(int MS, const StepArgs* table, const int2* m
   }
 }
 
+// The split form's kernels for window side MS (64 and more).
+cudaError_t split_launch_m(int MS, bool atomic, bool early, const StepArgs& a, int windows, cudaStream_t st) {
+  switch (MS) {
+    case 64: return split_launch<64>(atomic, early, a, windows, st);
+    case 128: return split_launch<128>(atomic, early, a, windows, st);
+    case 256: return split_launch<256>(atomic, early, a, windows, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+cudaError_t split_launch_batched_m(int MS, const StepArgs* table, const int2* map, int windows, cudaStream_t st) {
+  switch (MS) {
+    case 64: return split_launch_batched<64>(table, map, windows, st);
+    case 128: return split_launch_batched<128>(table, map, windows, st);
+    case 256: return split_launch_batched<256>(table, map, windows, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 // The three register bounds the autotuner tries for window side MS (c[3];
 // equal entries are one candidate).
 void minb_candidates(int MS, int* c) {
@@ -521,20 +557,20 @@ void minb_candidates(int MS, int* c) {
 }
 
 cudaError_t prepare_kernels(int MS) {
-  cudaError_t e = cudaFuncSetAttribute(apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)((sizeof(int2) + sizeof(int)) * kMaxMinibatch));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(apply_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((sizeof(int2) + sizeof(int)) * kMaxMinibatch));
+  cudaError_t e = cudaSuccess;
+  for (auto* k : {apply_kernel<16, 16>, apply_kernel<32, 32>, apply_tail_kernel})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(sizeof(ApplyEntry) * kMaxMinibatch));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(apply_kernel_batched<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((sizeof(int2) + sizeof(int)) * kMaxMinibatch));
+                             (int)(sizeof(ApplyEntry) * kMaxMinibatch));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(apply_kernel_batched<32, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((sizeof(int2) + sizeof(int)) * kMaxMinibatch));
+                             (int)(sizeof(ApplyEntry) * kMaxMinibatch));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(apply_kernel_batched<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((sizeof(int2) + sizeof(int)) * kMaxMinibatch));
+                             (int)(sizeof(ApplyEntry) * kMaxMinibatch));
   if (e == cudaSuccess && MS <= 128)
     e = cudaFuncSetAttribute(vcycle_up_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(2 * sizeof(float2) * (size_t)up_off(128, 8)));
@@ -567,6 +603,7 @@ struct GroupWindowLaunch {
   int ms;       // window side of this launch
   int map_off;  // first entry of its cluster map
   int windows;  // windows (clusters) in the launch
+  bool split;   // its members take the split form
 };
 struct GroupApplyLaunch {
   int tab_off;    // first entry of its problem table
@@ -778,6 +815,26 @@ StepArgs make_args(magpie_ctx* c, const int32_t* idx) {
   a.phase = (c->variant & 2) ? c->phase : nullptr;
   a.stamps = c->stamps;
   return a;
+}
+
+// Whether the context's minibatch steps take the split form of the window
+// phase: every plain or learned step with windows of 64 and more whose levels
+// fit a strip.  The probe step and the phase rule keep the cluster kernel.  us
+// per step, three levels, ordered update (split / cluster kernel):
+//   m = 64, n = 300   B = 16: 9.8 / 10.8, 64: 11.9 / 12.2, 128: 15.4 / 14.4, 512: 35.7 / 47.3
+//   m = 128, n = 512  B = 4: 11.3 / 14.9, 16: 14.9 / 16.7, 64: 20.7 / 22.0, 256: 57.8 / 66.7
+//   m = 256, n = 800  B = 4: 16.6 / 27.3, 16: 27.1 / 50.0, 64: 57.9 / 117
+// A function of the context alone, so that a member of a group takes the same
+// form as the context swept by itself (the objects are bitwise the same in
+// both forms, the FP64 sums of Phi_k and ||g|| are taken in another order).
+bool split_form(const magpie_ctx* c) {
+  const int m = c->p.m;
+  return m >= 64 && c->p.levels <= (m >= 128 ? Split<128>::LMAX : Split<64>::LMAX) && !c->p.update_probe &&
+         !c->precision && !(c->variant & 2) && !c->stamps;
+}
+// partial-sum slots per window its steps write
+int step_slots(const magpie_ctx* c) {
+  return c->precision ? c->p.m / kTcLines : split_form(c) ? c->p.m / Split<256>::NL : cluster_of(c->p.m);
 }
 
 // ------------------------------------------------- learned coarse correction
@@ -1238,13 +1295,21 @@ int enqueue_precision_g0(magpie_ctx* c, const int32_t* idx, int count, cudaStrea
 }
 
 // ev (optional): four events recorded before/after the window kernel and
-// before/after the apply kernel.
-int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, const cudaEvent_t* ev = nullptr) {
+// before/after the apply kernel.  own_idx: idx lies in the context's own
+// permutation, final before the stream's previous kernel began.
+int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, const cudaEvent_t* ev = nullptr,
+                 bool own_idx = false) {
   NvtxRange range("magpie minibatch step");
   StepArgs a = make_args(c, idx);
-  // the float-atomic update serves the FP32 window kernel without the phase
-  // rule or the learned correction; every other form uses the ordered one
-  const bool atom = c->acc && !c->precision && !c->cnn && !a.phase;
+  // the float-atomic update serves the FP32 window phase without the phase
+  // rule or the learned correction; every other form uses the ordered one, and
+  // so does the split form where that is the faster of the two: its gradient
+  // kernel waits for the atomics (m = 128, B = 64: 23.6 us per step against
+  // 21.0; m = 256, B = 64: 70.9 against 63.7; m = 64, B = 16: 10.3 against
+  // 9.8, B = 64: 11.8 against 11.9, B = 256: 20.5 against 21.7)
+  const bool split = split_form(c);
+  const bool atom = c->acc && !c->precision && !c->cnn && !a.phase &&
+                    (!split || (c->p.m == 64 && c->p.minibatch >= 64));
   if (ev) CUDA_TRY(cudaEventRecord(ev[0], st));
   int rc = MAGPIE_OK;
   if (c->precision) {
@@ -1260,7 +1325,10 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
     }
   } else {
     a.grad_only = c->cnn ? 1 : 0;
-    if (a.phase) {
+    if (split) {
+      if (atom) a.acc = c->acc;
+      CUDA_TRY(split_launch_m(c->p.m, atom, own_idx, a, count, st));
+    } else if (a.phase) {
       CUDA_TRY(launch_window_m<kStepRecycle>(c->p.m, a, count, st));
     } else if (atom) {
       a.acc = c->acc;
@@ -1277,7 +1345,7 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
     const size_t npix = (size_t)c->p.n_rows * c->p.n_cols;
     const unsigned blocks = (unsigned)std::min<size_t>((npix + 255) / 256, 152 * 8);
     CUDA_TRY(launch_ex(accum_apply_kernel, dim3(blocks), dim3(256), 0, st, 1, true, c->z, c->acc, npix, idx, count,
-                       c->p.n_pos, (const double*)c->part, cluster_of(c->p.m), c->p.m, c->phi_pos, c->gn_pos));
+                       c->p.n_pos, (const double*)c->part, step_slots(c), c->p.m, c->phi_pos, c->gn_pos));
   } else if (c->precision && !c->cnn && c->p.levels >= 2) {
     // contrib holds g^0 and g1buf e^1: the update forms w . Delta from them
     ApplyArgs P = apply_args(c->z, c->p.n_rows, c->p.n_cols, c->corner, idx, count, c->p.n_pos, c->contrib,
@@ -1286,18 +1354,17 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
     P.u0 = c->pyr;
     P.hand = c->hand;
     P.nhand = 3 * count;
-    const dim3 tiles(P.tiles_x, (c->p.n_rows + kApplyTile - 1) / kApplyTile);
-    CUDA_TRY(launch_ex(apply_tail_kernel, tiles, dim3(256), (sizeof(int2) + sizeof(int)) * count, st, 1, true, P));
+    CUDA_TRY(launch_ex(apply_tail_kernel, dim3((unsigned)apply_tiles(P)), dim3(256), sizeof(ApplyEntry) * count, st, 1,
+                       true, P));
   } else {
     ApplyArgs P = apply_args(c->z, c->p.n_rows, c->p.n_cols, c->corner, idx, count, c->p.n_pos, c->contrib,
-                             c->pyr + c->M, c->p.m, c->part, c->phi_pos, c->gn_pos,
-                             c->precision ? c->p.m / kTcLines : 0);
+                             c->pyr + c->M, c->p.m, c->part, c->phi_pos, c->gn_pos, step_slots(c));
     if (c->precision) {  // the transform kernels' hand-off counts
       P.hand = c->hand;
       P.nhand = 3 * count;
     }
-    const dim3 tiles(P.tiles_x, (c->p.n_rows + kApplyTile - 1) / kApplyTile);
-    CUDA_TRY(launch_ex(apply_kernel, tiles, dim3(256), (sizeof(int2) + sizeof(int)) * count, st, 1, true, P));
+    P.early = split ? 1 : 0;
+    CUDA_TRY(launch_apply_args(P, st));
   }
   if (c->p.update_probe) {
     probe_apply_kernel<<<(c->M + 255) / 256, 256, 0, st>>>(c->Q, c->M, idx, count, c->p.n_pos, c->pnum, c->pa2,
@@ -1367,7 +1434,7 @@ int capture_sweep(magpie_ctx* c, cudaGraphExec_t* out) {
   CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   int rc = MAGPIE_OK;
   for (int s = 0; s < N && rc == MAGPIE_OK; s += B)
-    rc = enqueue_step(c, c->order + s, N - s < B ? N - s : B, c->cap_stream);
+    rc = enqueue_step(c, c->order + s, N - s < B ? N - s : B, c->cap_stream, nullptr, true);
   cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
   if (rc) {
     if (g) cudaGraphDestroy(g);
@@ -1500,12 +1567,40 @@ int noalloc_scratch(NoAllocScratch* out) {
 }  // namespace magpie_impl
 
 
+// The window phase L of a batched step, the cluster kernel with register bound minb.
+cudaError_t launch_group_windows(magpie_group* g, const GroupWindowLaunch& L, cudaStream_t st, int minb) {
+  if (L.split) return split_launch_batched_m(L.ms, g->table, g->map + L.map_off, L.windows, st);
+  return launch_window_batched_m<kStep>(L.ms, g->table, g->map + L.map_off, L.windows, st, minb);
+}
+
+// The window phases of batched step t: the window sides run concurrently,
+// forked from `st` onto the group's side streams and joined back (a group of
+// 12 uneven problems: 2.74 ms per sweep, the sides one after another 2.96).
+int enqueue_group_windows(magpie_group* g, size_t t, cudaStream_t st) {
+  const auto& Ls = g->wl[t];
+  bool several = false;
+  for (const auto& L : Ls) several |= L.ms != Ls[0].ms;
+  if (several) CUDA_TRY(cudaEventRecord(g->fork, st));
+  int j = 0;  // side streams in the order of the window sides
+  for (size_t i = 0; i < Ls.size(); ++i) {
+    if (i && Ls[i].ms != Ls[i - 1].ms) ++j;
+    cudaStream_t s = j == 0 ? st : g->side[j];
+    if (j && Ls[i].ms != Ls[i - 1].ms) CUDA_TRY(cudaStreamWaitEvent(s, g->fork, 0));
+    CUDA_TRY(launch_group_windows(g, Ls[i], s, g->minb[ilog2(Ls[i].ms) - 3]));
+    if (j && (i + 1 == Ls.size() || Ls[i + 1].ms != Ls[i].ms)) {
+      CUDA_TRY(cudaEventRecord(g->join[j], s));
+      CUDA_TRY(cudaStreamWaitEvent(st, g->join[j], 0));
+    }
+  }
+  return MAGPIE_OK;
+}
+
 // The update of batched step t with apply tile shape v, from the device table
 // `table` (default: the group's own table of that shape).
 cudaError_t launch_apply_batched(magpie_group* g, int v, int t, cudaStream_t st, const ApplyArgs* table = nullptr) {
   const GroupApplyLaunch& A = g->al[v][t];
   const ApplyArgs* tab = table ? table : g->atable[v] + A.tab_off;
-  const size_t smem = (sizeof(int2) + sizeof(int)) * A.max_count;
+  const size_t smem = sizeof(ApplyEntry) * A.max_count;
   switch (v) {
     case 0: apply_kernel_batched<16, 16><<<A.blocks, 256, smem, st>>>(tab, A.n); break;
     case 1: apply_kernel_batched<32, 8><<<A.blocks, 256, smem, st>>>(tab, A.n); break;
@@ -1639,11 +1734,8 @@ int group_tune_form(magpie_group* g, cudaStream_t st, cudaEvent_t e0, cudaEvent_
   if (e == cudaSuccess) e = cudaMemcpyAsync(ptab, pt.data(), sizeof(ApplyArgs) * pt.size(), cudaMemcpyHostToDevice, st);
   auto run = [&](int form) -> int {
     if (form == 0) {
-      for (const auto& L : g->wl[0]) {
-        cudaError_t le = launch_window_batched_m<kStep>(L.ms, g->table, g->map + L.map_off, L.windows, st,
-                                                        g->minb[ilog2(L.ms) - 3]);
-        if (le != cudaSuccess) return fail(MAGPIE_ECUDA, std::string("group autotuner: ") + cudaGetErrorString(le));
-      }
+      const int wrc = enqueue_group_windows(g, 0, st);
+      if (wrc) return wrc;
       CUDA_TRY(launch_apply_batched(g, g->apply_shape, 0, st, atab));
       return MAGPIE_OK;
     }
@@ -1669,7 +1761,12 @@ int group_tune_form(magpie_group* g, cudaStream_t st, cudaEvent_t e0, cudaEvent_
   if (rc) return rc;
   if (e != cudaSuccess) return fail(MAGPIE_ECUDA, std::string("group autotuner (form): ") + cudaGetErrorString(e));
   if (h) return fail(MAGPIE_ETIMEOUT, "group autotuner: a dependency wait of the persistent form ran out");
-  g->persistent = g->form_ms[1] < g->form_ms[0] ? 1 : 0;
+  // a member whose sweeps take the split form gets the same FP64 window sums
+  // from the group only in separate launches (the persistent form runs the
+  // cluster kernel)
+  bool split = false;
+  for (const auto* c : g->members) split |= split_form(c);
+  g->persistent = !split && g->form_ms[1] < g->form_ms[0] ? 1 : 0;
   return MAGPIE_OK;
 }
 
@@ -1695,6 +1792,7 @@ int group_autotune(magpie_group* g) {
   if (!g->wl.empty())
     for (const auto& L : g->wl[0]) {
       if (e != cudaSuccess) break;
+      // (for a side in the split form the bound serves the persistent form)
       const int i = ilog2(L.ms) - 3;
       int cand[3];
       minb_candidates(L.ms, cand);
@@ -2140,30 +2238,34 @@ int magpie_group_create(magpie_group** out, magpie_ctx* const* ctxs, int32_t n, 
     std::vector<GroupWindowLaunch> wls;
     std::vector<GroupPersistLaunch> pls;
     for (int ms : {8, 16, 32, 64, 128, 256}) {
-      GroupWindowLaunch L{ms, (int)map.size(), 0};
       GroupPersistLaunch PL{ms, (int)map.size(), 0, (int)g->ptable_host.size(), 0, 0, q_total, 0, 0};
       const int pt = window_threads(ms) >= 256 ? 32 : 16;  // the persistent kernel's update tile
-      for (int i = 0; i < n; ++i) {
-        magpie_ctx* c = g->members[i];
-        if (entry[i] < 0 || c->p.m != ms) continue;
-        const int cnt = std::min(c->p.minibatch, c->p.n_pos - t * c->p.minibatch);
-        for (int w = 0; w < cnt; ++w) {
-          map.push_back(make_int2(entry[i], w));
-          wmem.push_back(PL.na);
+      // the members of the cluster kernel, then those of the split form: one
+      // window launch each, one item list of the persistent form for both
+      for (const bool split : {false, true}) {
+        GroupWindowLaunch L{ms, (int)map.size(), 0, split};
+        for (int i = 0; i < n; ++i) {
+          magpie_ctx* c = g->members[i];
+          if (entry[i] < 0 || c->p.m != ms || split_form(c) != split) continue;
+          const int cnt = std::min(c->p.minibatch, c->p.n_pos - t * c->p.minibatch);
+          for (int w = 0; w < cnt; ++w) {
+            map.push_back(make_int2(entry[i], w));
+            wmem.push_back(PL.na);
+          }
+          L.windows += cnt;
+          ApplyArgs P = apply_args(c->z, c->p.n_rows, c->p.n_cols, c->corner, c->order + (size_t)t * c->p.minibatch,
+                                   cnt, c->p.n_pos, c->contrib, c->pyr + c->M, c->p.m, c->part, c->phi_pos,
+                                   c->gn_pos, 0, ApplyShape{pt, pt});
+          P.block0 = PL.ntiles;
+          PL.ntiles += apply_tiles(P);
+          PL.max_count = std::max(PL.max_count, cnt);
+          ++PL.na;
+          g->ptable_host.push_back(P);
         }
-        L.windows += cnt;
-        ApplyArgs P = apply_args(c->z, c->p.n_rows, c->p.n_cols, c->corner, c->order + (size_t)t * c->p.minibatch,
-                                 cnt, c->p.n_pos, c->contrib, c->pyr + c->M, c->p.m, c->part, c->phi_pos,
-                                 c->gn_pos, 0, ApplyShape{pt, pt});
-        P.block0 = PL.ntiles;
-        PL.ntiles += apply_tiles(P);
-        PL.max_count = std::max(PL.max_count, cnt);
-        ++PL.na;
-        g->ptable_host.push_back(P);
+        if (L.windows) wls.push_back(L);
+        PL.nw += L.windows;
       }
-      if (L.windows) {
-        wls.push_back(L);
-        PL.nw = L.windows;
+      if (PL.nw) {
         q_total += 1 + PL.na;
         pls.push_back(PL);
       }
@@ -2180,7 +2282,7 @@ int magpie_group_create(magpie_group** out, magpie_ctx* const* ctxs, int32_t n, 
         const int cnt = std::min(c->p.minibatch, c->p.n_pos - t * c->p.minibatch);
         ApplyArgs P = apply_args(c->z, c->p.n_rows, c->p.n_cols, c->corner, c->order + (size_t)t * c->p.minibatch,
                                  cnt, c->p.n_pos, c->contrib, c->pyr + c->M, c->p.m, c->part, c->phi_pos,
-                                 c->gn_pos, 0, kApplyShapes[v]);
+                                 c->gn_pos, step_slots(c), kApplyShapes[v]);
         P.block0 = A.blocks;
         A.blocks += apply_tiles(P);
         A.max_count = std::max(A.max_count, cnt);
@@ -2255,14 +2357,9 @@ int magpie_group_sweep(magpie_group* g, const int32_t* const* orders) {
       for (size_t t = 0; t < g->pl.size() && e == cudaSuccess && !rc; ++t)
         rc = enqueue_persistent_step(g, t, g->cap_stream, g->ptable, 0);
     } else {
-      for (size_t t = 0; t < g->wl.size() && e == cudaSuccess; ++t) {
-        for (const auto& L : g->wl[t]) {
-          e = launch_window_batched_m<kStep>(L.ms, g->table, g->map + L.map_off, L.windows, g->cap_stream,
-                                             g->minb[ilog2(L.ms) - 3]);
-          if (e != cudaSuccess) break;
-        }
-        if (e != cudaSuccess) break;
-        e = launch_apply_batched(g, g->apply_shape, t, g->cap_stream);
+      for (size_t t = 0; t < g->wl.size() && e == cudaSuccess && !rc; ++t) {
+        rc = enqueue_group_windows(g, t, g->cap_stream);
+        if (!rc) e = launch_apply_batched(g, g->apply_shape, t, g->cap_stream);
       }
     }
     cudaError_t e2 = cudaStreamEndCapture(g->cap_stream, &gr);

@@ -5,17 +5,15 @@
 
 // z += sum_b contrib_b / sum_b w0 over the windows covering each pixel, in
 // minibatch order (bitwise reproducible).  One block of NT (256) threads per
-// 16 x 16 object tile, one pixel per thread: the block first lists, in
-// minibatch order, the windows that overlap its tile (corners as recorded by
-// the window kernel; a ballot compaction over all warps); each thread then
-// walks that short list four entries at a time with predicated loads, so
-// several increments are in flight per thread.  Block (0, 0) also turns the
-// window kernel's block partials into Phi_k and ||grad Phi_k||.
-// Dynamic smem: count int2 corners + count ints.  The tile is TW x TH pixels
-// (16 x 16 for single problems; the group autotuner also tries 32 x 8 and
-// 32 x 32, four pixels per thread); every shape sums each pixel's windows in
-// minibatch order, so all give bitwise equal objects.
-constexpr int kApplyTile = 16;
+// TW x TH object tile, TW TH / NT pixels of one column per thread: the block
+// first lists, in minibatch order, the windows that overlap its tile (corners
+// as recorded by the window kernel; a ballot compaction over all warps), each
+// with its increments' offset; each thread then walks that list a few entries
+// at a time with predicated loads, so several increments are in flight per
+// thread.  The block after the last tile turns the window kernel's block
+// partials into Phi_k and ||grad Phi_k||, beside the tiles rather than before
+// one of them.  Dynamic smem: count entries.  Every tile shape sums each
+// pixel's windows in minibatch order, so all give bitwise equal objects.
 struct ApplyShape {
   int tw, th;
 };
@@ -42,99 +40,126 @@ struct ApplyArgs {
   const float* u0;         // [MS][MS] u^0
   int* hand;               // precision form: the step's window hand-off counts, zeroed by
   int nhand;               // block (0, 0) once the grid may run (null otherwise)
+  int early;               // the object and the corners are final before the stream's previous kernel
+                           // ends (split form): the windows are listed before the wait for it
 };
+
+// One window of a tile's list: its corner, the offset of its increments less
+// that of its corner (so that pixel (r, c) is at off + r MS + c), its slot.
+struct ApplyEntry {
+  int qx, qy, off, b;
+};
+
+// Phi_k and ||grad Phi_k|| of the step's windows from the block partials, in block order.
+__device__ __forceinline__ void apply_partials(const ApplyArgs& P) {
+  for (int b = threadIdx.x; b < P.count; b += blockDim.x) {
+    const int k = P.idx[b];
+    if ((unsigned)k >= (unsigned)P.n_pos) continue;
+    double a = 0.0, g = 0.0;
+    for (int q = 0; q < P.slots; ++q) {
+      a += P.part[(size_t)(b * P.slots + q) * 2];
+      g += P.part[(size_t)(b * P.slots + q) * 2 + 1];
+    }
+    P.phi_pos[k] = a / (2.0 * (double)P.MS * (double)P.MS);
+    P.gn_pos[k] = sqrt(g);
+  }
+}
 
 template <int TW, int TH, int NT = 256, bool TAIL = false>
 __device__ __forceinline__ void apply_body(const ApplyArgs& P, const int tx, const int ty) {
   static_assert((TW * TH) % NT == 0 && NT % TW == 0 && NT % 32 == 0, "NT threads cover the tile in whole rows");
   constexpr int PPT = TW * TH / NT, RS = NT / TW, NW = NT / 32;  // pixels per thread, rows per pass, warps
-  extern __shared__ int2 corner[];
-  const int count = P.count, MS = P.MS;
-  int* list = reinterpret_cast<int*>(corner + count);
-  __shared__ int warp_hits[NW], n_list;
-  if (tx == 0 && ty == 0) {
-    // the window kernel's block partials -> Phi_k and ||grad Phi_k||, in block order
-    for (int b = threadIdx.x; b < count; b += blockDim.x) {
-      const int k = P.idx[b];
-      if ((unsigned)k >= (unsigned)P.n_pos) continue;
-      double a = 0.0, g = 0.0;
-      for (int q = 0; q < P.slots; ++q) {
-        a += P.part[(size_t)(b * P.slots + q) * 2];
-        g += P.part[(size_t)(b * P.slots + q) * 2 + 1];
-      }
-      P.phi_pos[k] = a / (2.0 * (double)MS * (double)MS);
-      P.gn_pos[k] = sqrt(g);
+  constexpr int U = PPT >= 4 ? 2 : kApplyUnroll;                  // list entries in flight
+  extern __shared__ __align__(16) unsigned char apply_smem[];
+  ApplyEntry* list = reinterpret_cast<ApplyEntry*>(apply_smem);
+  __shared__ int warp_hits[NW];
+  if (!P.early) grid_dep_wait();
+  if (ty >= P.tiles_y) {  // the block after the last tile
+    if (P.early) {
+      grid_dep_wait();
+      grid_dep_launch();
     }
+    apply_partials(P);
+    return;
   }
+  const int count = P.count, MS = P.MS, M = MS * MS;
   const int R0 = ty * TH, C0 = tx * TW;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int r0 = R0 + (int)(threadIdx.x / TW), c = C0 + (int)(threadIdx.x % TW);
+  float2 zz[PPT];
+#pragma unroll
+  for (int p = 0; p < PPT; ++p)
+    zz[p] = (r0 + p * RS < P.n_rows && c < P.n_cols) ? __ldcg(&P.z[(size_t)(r0 + p * RS) * P.n_cols + c])
+                                                      : make_float2(0.f, 0.f);
   // windows meeting this tile, listed in minibatch order: every warp takes
   // 32 consecutive windows per round, ballots, and the rounds are stitched
   // together by per-warp counts
-  int base = 0;
+  int nl = 0;
   for (int b0 = 0; b0 < count; b0 += NT) {
     const int b = b0 + threadIdx.x;
     bool hit = false;
+    int2 q = make_int2(0, 0);
     if (b < count) {
-      const int2 q = P.corners[b];
-      corner[b] = q;
+      q = __ldcg(&P.corners[b]);
       hit = q.x < R0 + TH && q.x + MS > R0 && q.y < C0 + TW && q.y + MS > C0;
     }
     const unsigned mask = __ballot_sync(0xffffffffu, hit);
     if (lane == 0) warp_hits[wid] = __popc(mask);
     __syncthreads();
-    int off = base;
-    for (int i = 0; i < wid; ++i) off += warp_hits[i];
-    if (hit) list[off + __popc(mask & ((1u << lane) - 1u))] = b;
-    int tot = 0;
-    for (int i = 0; i < NW; ++i) tot += warp_hits[i];
-    base += tot;
+    int off = nl;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+      if (i < wid) off += warp_hits[i];
+      nl += warp_hits[i];
+    }
+    if (hit) list[off + __popc(mask & ((1u << lane) - 1u))] = ApplyEntry{q.x, q.y, b * M - q.x * MS - q.y, b};
     __syncthreads();
   }
-  if (threadIdx.x == 0) n_list = base;
-  __syncthreads();
-  const int nl = n_list;
-  const size_t M = (size_t)MS * MS;
-#pragma unroll 1
-  for (int pp = 0; pp < PPT; ++pp) {
-    const int r = R0 + (int)(threadIdx.x / TW) + pp * RS, c = C0 + (int)(threadIdx.x % TW);
-    if (r >= P.n_rows || c >= P.n_cols) continue;
-    float nx = 0.f, ny = 0.f, d = 0.f;
-    for (int j0 = 0; j0 < nl; j0 += kApplyUnroll) {
-      float2 v[kApplyUnroll];
-      float wv[kApplyUnroll];
+  if (P.early) {
+    grid_dep_wait();
+    grid_dep_launch();
+  }
+  float nx[PPT], ny[PPT], d[PPT];
 #pragma unroll
-      for (int u = 0; u < kApplyUnroll; ++u) {
-        const int j = j0 + u;
-        const int b = j < nl ? list[j] : 0;
-        const int2 q = corner[b];
-        const int dr = r - q.x, dc = c - q.y;
-        const bool in = j < nl && (unsigned)dr < (unsigned)MS && (unsigned)dc < (unsigned)MS;
-        const int o = in ? dr * MS + dc : 0;
-        v[u] = in ? P.contrib[(size_t)b * M + o] : make_float2(0.f, 0.f);
-        wv[u] = in ? __ldg(&P.w0[o]) : 0.f;
+  for (int p = 0; p < PPT; ++p) nx[p] = ny[p] = d[p] = 0.f;
+  const int o0 = r0 * MS + c;
+#pragma unroll 1
+  for (int j0 = 0; j0 < nl; j0 += U) {
+    float2 v[U][PPT];
+    float wv[U][PPT];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool live = j0 + u < nl;
+      const ApplyEntry q = list[live ? j0 + u : 0];
+      const bool inc = live && (unsigned)(c - q.qy) < (unsigned)MS;
+      const int qo = q.qx * MS + q.qy;
+#pragma unroll
+      for (int p = 0; p < PPT; ++p) {
+        const int dr = r0 + p * RS - q.qx;
+        const bool in = inc && (unsigned)dr < (unsigned)MS;
+        const int o = o0 + p * RS * MS;
+        v[u][p] = in ? __ldcg(&P.contrib[q.off + o]) : make_float2(0.f, 0.f);
+        wv[u][p] = in ? __ldg(&P.w0[o - qo]) : 0.f;
         if constexpr (TAIL) {
           // w . Delta = g^0 + u^0 e^1 at this window pixel, e^1 of its 2 x 2 bin
-          const int h = MS >> 1;
-          const float2 e = in ? P.e1[(size_t)b * h * h + (dr >> 1) * h + (dc >> 1)] : make_float2(0.f, 0.f);
-          const float uo = in ? __ldg(&P.u0[o]) : 0.f;
-          v[u] = make_float2(__fmaf_rn(uo, e.x, v[u].x), __fmaf_rn(uo, e.y, v[u].y));
+          const int h = MS >> 1, dc = c - q.qy;
+          const float2 e = in ? P.e1[q.b * h * h + (dr >> 1) * h + (dc >> 1)] : make_float2(0.f, 0.f);
+          const float uo = in ? __ldg(&P.u0[o - qo]) : 0.f;
+          v[u][p] = make_float2(__fmaf_rn(uo, e.x, v[u][p].x), __fmaf_rn(uo, e.y, v[u][p].y));
         }
       }
+    }
 #pragma unroll
-      for (int u = 0; u < kApplyUnroll; ++u) {
-        nx += v[u].x;
-        ny += v[u].y;
-        d += wv[u];
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int p = 0; p < PPT; ++p) {
+        nx[p] += v[u][p].x;
+        ny[p] += v[u][p].y;
+        d[p] += wv[u][p];
       }
-    }
-    if (d > 0.f) {
-      const size_t p = (size_t)r * P.n_cols + c;
-      float2 zz = P.z[p];
-      zz.x += nx / d;
-      zz.y += ny / d;
-      P.z[p] = zz;
-    }
   }
+#pragma unroll
+  for (int p = 0; p < PPT; ++p)
+    if (d[p] > 0.f)  // only pixels of the object have windows
+      P.z[(size_t)(r0 + p * RS) * P.n_cols + c] = make_float2(zz[p].x + nx[p] / d[p], zz[p].y + ny[p] / d[p]);
 }
-

@@ -5,4 +5,5 @@
 
 namespace magpie_impl {
 MAGPIE_INSTANTIATE_WINDOW(128)
+MAGPIE_INSTANTIATE_SPLIT(128)
 }  // namespace magpie_impl

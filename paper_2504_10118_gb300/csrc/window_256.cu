@@ -5,4 +5,5 @@
 
 namespace magpie_impl {
 MAGPIE_INSTANTIATE_WINDOW(256)
+MAGPIE_INSTANTIATE_SPLIT(256)
 }  // namespace magpie_impl

@@ -5,4 +5,5 @@
 
 namespace magpie_impl {
 MAGPIE_INSTANTIATE_WINDOW(64)
+MAGPIE_INSTANTIATE_SPLIT(64)
 }  // namespace magpie_impl

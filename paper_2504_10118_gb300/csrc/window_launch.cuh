@@ -62,7 +62,7 @@ void window_minb_candidates(int* c) {
 
 template <int MS>
 size_t persistent_smem(int max_count) {
-  return std::max(Geo<MS>::SMEM, (sizeof(int2) + sizeof(int)) * (size_t)max_count);
+  return std::max(Geo<MS>::SMEM, sizeof(ApplyEntry) * (size_t)max_count);
 }
 
 template <int MS>
@@ -139,6 +139,33 @@ cudaError_t window_prepare() {
                              pbytes);
   return e;
 }
+
+// The three kernels of the split form, each a programmatic dependent of the
+// one before (the exit kernel of the stream's previous kernel).
+template <int MS>
+cudaError_t split_launch(bool atomic, bool early, const StepArgs& a, int windows, cudaStream_t st) {
+  using S = Split<MS>;
+  const dim3 grid((unsigned)windows * S::TILES), block(S::T);
+  cudaError_t e = launch_ex(split_exit_kernel<MS>, grid, block, 0, st, 1, true, a, early);
+  if (e == cudaSuccess) e = launch_ex(split_project_kernel<MS>, grid, block, 0, st, 1, true, a);
+  if (e == cudaSuccess)
+    e = launch_ex(atomic ? split_grad_kernel<MS, true> : split_grad_kernel<MS, false>, grid, block, 0, st, 1, true, a);
+  return e;
+}
+
+template <int MS>
+cudaError_t split_launch_batched(const StepArgs* table, const int2* map, int windows, cudaStream_t st) {
+  using S = Split<MS>;
+  const dim3 grid((unsigned)windows * S::TILES), block(S::T);
+  cudaError_t e = launch_ex(split_kernel_batched<MS, 0>, grid, block, 0, st, 1, false, table, map);
+  if (e == cudaSuccess) e = launch_ex(split_kernel_batched<MS, 1>, grid, block, 0, st, 1, true, table, map);
+  if (e == cudaSuccess) e = launch_ex(split_kernel_batched<MS, 2>, grid, block, 0, st, 1, true, table, map);
+  return e;
+}
+
+#define MAGPIE_INSTANTIATE_SPLIT(S)                                                     \
+  template cudaError_t split_launch<S>(bool, bool, const StepArgs&, int, cudaStream_t); \
+  template cudaError_t split_launch_batched<S>(const StepArgs*, const int2*, int, cudaStream_t);
 
 #define MAGPIE_INSTANTIATE_WINDOW(S)                                                                       \
   template cudaError_t window_launch<S>(int, const StepArgs&, int, cudaStream_t);                          \
