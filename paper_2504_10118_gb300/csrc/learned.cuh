@@ -362,120 +362,6 @@ __global__ void __launch_bounds__(256) conv_splitk_kernel(const ConvFwd a, int s
   }
 }
 
-// --------------------------------------------------------- backward (FP32)
-// dx[b, iy, ix, ci] = sum over the outputs that read (iy, ix) of
-// dz[b, oy, ox, co] W[co, ky, kx, ci], then the previous layer's ReLU mask.
-__global__ void __launch_bounds__(256) conv_bwd_data_kernel(const float* __restrict__ dz, const bf16* __restrict__ w,
-                                                            const bf16* __restrict__ a_prev, float* __restrict__ dx,
-                                                            int B, int Hin, int Cin, int Cout, int stride, int up,
-                                                            int Ho) {
-  const size_t n = (size_t)B * Hin * Hin * Cin;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int ci = (int)(e % Cin);
-    const size_t pix = e / Cin;
-    const int ix = (int)(pix % Hin), iy = (int)((pix / Hin) % Hin), b = (int)(pix / ((size_t)Hin * Hin));
-    float acc = 0.f;
-    if (__bfloat162float(a_prev[e]) > 0.f) {
-      for (int uy = 0; uy < up; ++uy)
-        for (int ky = 0; ky < 3; ++ky) {
-          const int ty = iy * up + uy + 1 - ky;
-          if (ty < 0 || ty % stride) continue;
-          const int oy = ty / stride;
-          if (oy >= Ho) continue;
-          for (int ux = 0; ux < up; ++ux)
-            for (int kx = 0; kx < 3; ++kx) {
-              const int tx = ix * up + ux + 1 - kx;
-              if (tx < 0 || tx % stride) continue;
-              const int ox = tx / stride;
-              if (ox >= Ho) continue;
-              const float* d = dz + ((size_t)(b * Ho + oy) * Ho + ox) * Cout;
-              const bf16* wp = w + (size_t)(ky * 3 + kx) * Cin + ci;
-              for (int co = 0; co < Cout; ++co) acc += d[co] * __bfloat162float(wp[(size_t)co * 9 * Cin]);
-            }
-        }
-    }
-    dx[e] = acc;
-  }
-}
-
-// Weight and bias gradients of one layer as an FP32 GEMM over the output
-// pixels p: dW[co][k] = sum_p dz[p][co] A[p][k], where A is the forward
-// pass's gather (k < K = 9 Cin) and A[p][K] = 1 (the bias column).  Block:
-// 64 channels x 64 k, 256 threads with 4 x 4 results each, 16 pixels per
-// shared-memory stage; the pixel range is split over gridDim.z (chunks of
-// `chunk` pixels) into partial sums part[z][param] (weights, then biases).
-__global__ void __launch_bounds__(256) conv_wgrad_kernel(const float* __restrict__ dz, const bf16* __restrict__ a_in,
-                                                         float* __restrict__ part, int B, int Hin, int Cin, int Cout,
-                                                         int stride, int up, int Ho, int chunk) {
-  __shared__ float Ds[16][64];
-  __shared__ float As[16][64];
-  const int K = 9 * Cin, Kb = K + 1, P = Cout * K + Cout;
-  const int co0 = blockIdx.y * 64, k0 = blockIdx.x * 64;
-  const int npix = B * Ho * Ho;
-  const int p0 = blockIdx.z * chunk, p1 = min(npix, p0 + chunk);
-  const int Hv = Hin * up;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int pb = p0; pb < p1; pb += 16) {
-    for (int i = threadIdx.x; i < 16 * 64; i += 256) {
-      const int pp = i / 64, c = i % 64;
-      const int p = pb + pp, co = co0 + c, k = k0 + c;
-      Ds[pp][c] = (p < p1 && co < Cout) ? dz[(size_t)p * Cout + co] : 0.f;
-      float av = 0.f;
-      if (p < p1 && k < Kb) {
-        if (k == K) {
-          av = 1.f;
-        } else {
-          const int tap = k / Cin, ci = k - tap * Cin;
-          const int ky = tap / 3, kx = tap - 3 * ky;
-          const int b = p / (Ho * Ho), r2 = p - b * Ho * Ho;
-          const int oy = r2 / Ho, ox = r2 - oy * Ho;
-          const int vy = oy * stride + ky - 1, vx = ox * stride + kx - 1;
-          if (vy >= 0 && vy < Hv && vx >= 0 && vx < Hv)
-            av = __bfloat162float(a_in[((size_t)(b * Hin + vy / up) * Hin + vx / up) * Cin + ci]);
-        }
-      }
-      As[pp][c] = av;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int pp = 0; pp < 16; ++pp) {
-      float d[4], a[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        d[j] = Ds[pp][ty * 4 + j];
-        a[j] = As[pp][tx * 4 + j];
-      }
-#pragma unroll
-      for (int i2 = 0; i2 < 4; ++i2)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i2][j] += d[i2] * a[j];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i2 = 0; i2 < 4; ++i2)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int co = co0 + ty * 4 + i2, k = k0 + tx * 4 + j;
-      if (co < Cout && k < Kb) part[(size_t)blockIdx.z * P + (k < K ? co * K + k : Cout * K + co)] = acc[i2][j];
-    }
-}
-
-// grad[p] = sum over chunks of part[chunk][p], in chunk order.
-__global__ void __launch_bounds__(256) chunk_sum_kernel(const float* __restrict__ part, float* __restrict__ grad, int P,
-                                                        int chunks) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  float s = 0.f;
-  for (int c = 0; c < chunks; ++c) s += part[(size_t)c * P + p];
-  grad[p] = s;
-}
-
 // --------------------------------------------------------------- training
 // L = 1/2 mean((y - t)^2) with t = (z_H^T - z_H^0) / s - e_plain / s taken
 // from the input x0 = (z_H^0, e_plain / s), the later z_H^T and s; dy = (y - t) / n.

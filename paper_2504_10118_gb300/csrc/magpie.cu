@@ -54,6 +54,7 @@ namespace magpie_impl {
 constexpr int kVersion = 10300;  // 1.3.0
 
 #include "learned.cuh"
+#include "learned_backward.cuh"
 #include "umma.cuh"
 #include "precision.cuh"
 
@@ -905,22 +906,40 @@ ConvPlan conv_plan_tc(const ConvFwd& a) {
   return pl;
 }
 
-// Pixel chunks of the weight-gradient GEMM of layer l (enough blocks to
-// fill the GPU, at least 64 pixels per chunk).
-struct WgradPlan {
-  int gx, gy, chunks, chunk;
+// Split of a batch's backward pass: per layer 1 .. 4 the weight gradient's
+// tiles and pixel chunks (enough blocks for two per SM, at least 128 pixels
+// per chunk), the blocks of layers 0 and 5, and where each keeps its partial
+// sums.
+struct GradPlan {
+  int wm[kCnnLayers], wn[kCnnLayers], chunk[kCnnLayers], chunks[kCnnLayers];
+  size_t stride[kCnnLayers], off[kCnnLayers], floats;
 };
-WgradPlan wgrad_plan(int h, int l, int B) {
-  const CnnLayer& L = kCnn[l];
-  const int Ho = cnn_side_out(h, l), npix = B * Ho * Ho;
-  WgradPlan w{};
-  w.gx = (9 * L.cin + 1 + 63) / 64;
-  w.gy = (L.cout + 63) / 64;
-  const int want = std::max(1, (2 * 152 + w.gx * w.gy - 1) / (w.gx * w.gy));
-  w.chunks = std::max(1, std::min(want, npix / 64));
-  w.chunk = (npix + w.chunks - 1) / w.chunks;
-  w.chunks = (npix + w.chunk - 1) / w.chunk;
-  return w;
+GradPlan grad_plan(int h, int B) {
+  GradPlan g{};
+  for (int l = 0; l < kCnnLayers; ++l) {
+    const CnnLayer& L = kCnn[l];
+    const int hi = cnn_side_in(h, l), ho = cnn_side_out(h, l);
+    if (l == 0) {
+      g.chunks[l] = std::min(2 * 152, (B * ho * ho + 63) / 64);
+      g.stride[l] = kFirstPart;
+    } else if (l == kCnnLayers - 1) {
+      g.chunks[l] = std::min(2 * 152, (B * hi * hi + kLastQ - 1) / kLastQ);
+      g.stride[l] = kLastPart;
+    } else {
+      const bool up = L.up > 1;
+      const int M = up ? 9 * L.cout : L.cout, N = up ? L.cin : 9 * L.cin, K = B * (up ? hi * hi : ho * ho);
+      g.wm[l] = M / 64;
+      g.wn[l] = (N + 63) / 64;
+      const int tiles = g.wm[l] * g.wn[l];
+      const int want = std::max(1, std::min((2 * 152 + tiles - 1) / tiles, K / 128));
+      g.chunk[l] = ((K + want - 1) / want + 31) / 32 * 32;
+      g.chunks[l] = (K + g.chunk[l] - 1) / g.chunk[l];
+      g.stride[l] = (size_t)M * N + M;
+    }
+    g.off[l] = g.floats;
+    g.floats += (g.stride[l] * g.chunks[l] + 3) / 4 * 4;
+  }
+  return g;
 }
 
 // Partial-sum floats needed by any batch of 1 .. max_batch windows.
@@ -941,9 +960,8 @@ size_t cnn_part_floats(int h, int max_batch) {
       const ConvPlan pt = conv_plan_tc(a);
       if (pt.splits > 1) n = std::max(n, (size_t)pt.splits * B * Ho * Ho * a.Cout);
     }
-    const int P = a.Cout * 9 * a.Cin + a.Cout;
-    n = std::max(n, (size_t)wgrad_plan(h, l, B).chunks * P);
   }
+  for (int B = 1; B <= max_batch; ++B) n = std::max(n, grad_plan(h, B).floats);
   return n;
 }
 
@@ -1009,30 +1027,89 @@ int cnn_enqueue_forward(magpie_cnn* n, const float* x, int batch, float* y, cuda
   return MAGPIE_OK;
 }
 
-// Gradient of <dy, y> over the parameters, for the inputs of the last forward pass.
+// Gradient of <dy, y> over the parameters, for the inputs of the last forward
+// pass (learned_backward.cuh).  dz[1] holds dz4, then dz3 behind it, then dz1;
+// dz[0] holds S of layer 4, dz2 behind it, then dz0.
 int cnn_enqueue_backward(magpie_cnn* n, const float* dy, float* grad, cudaStream_t st) {
   const int h = n->h, B = n->last_batch;
-  const float* dz = dy;
-  int cur = 0;
-  for (int l = kCnnLayers - 1; l >= 0; --l) {
+  const GradPlan g = grad_plan(h, B);
+  const auto pixels = [&](int l) { return (size_t)B * cnn_side_in(h, l) * cnn_side_in(h, l); };  // of layer l's input
+  const int last = kCnnLayers - 1;
+  float* dz4 = n->dz[1];
+  grad_last_kernel<<<g.chunks[last], 256, 0, st>>>(dy, n->wbf + n->off[last], n->act[last], dz4, n->part + g.off[last],
+                                                   (int)pixels(last), ilog2(cnn_side_in(h, last)));
+  CUDA_TRY(cudaGetLastError());
+  uint16_t* planes[kCnnLayers] = {};  // planes of dz (layers 3, 2, 1) and of layer 4's S
+  planes[4] = reinterpret_cast<uint16_t*>(n->dz[0]);
+  planes[3] = reinterpret_cast<uint16_t*>(dz4 + pixels(5) * kCnn[4].cout);
+  planes[2] = planes[4] + 3 * pixels(4) * 9 * kCnn[4].cout;
+  planes[1] = reinterpret_cast<uint16_t*>(n->dz[1]);
+  const size_t s4 = pixels(4) * 9 * kCnn[4].cout;
+  grad_sum4_kernel<<<(unsigned)((pixels(4) * 64 + 255) / 256), 256, 0, st>>>(dz4, planes[4], s4, (int)pixels(4),
+                                                                             ilog2(cnn_side_in(h, 4)));
+  CUDA_TRY(cudaGetLastError());
+  for (int l = 4; l >= 1; --l) {
     const CnnLayer& L = kCnn[l];
-    const int Hin = cnn_side_in(h, l), Ho = cnn_side_out(h, l);
-    const int P = L.cout * 9 * L.cin + L.cout;
-    const WgradPlan wp = wgrad_plan(h, l, B);
-    conv_wgrad_kernel<<<dim3(wp.gx, wp.gy, wp.chunks), 256, 0, st>>>(dz, n->act[l], n->part, B, Hin, L.cin, L.cout,
-                                                                      L.stride, L.up, Ho, wp.chunk);
+    const bool up = L.up > 1;
+    const int hi = cnn_side_in(h, l), ho = cnn_side_out(h, l);
+    GradGemm a{};
+    a.d = planes[l];
+    a.dplane = up ? s4 : (size_t)B * ho * ho * L.cout;
+    a.act = n->act[l];
+    a.part = n->part + g.off[l];
+    a.M = up ? 9 * L.cout : L.cout;
+    a.N = up ? L.cin : 9 * L.cin;
+    a.K = (int)(up ? pixels(l) : (size_t)B * ho * ho);
+    a.chunk = g.chunk[l];
+    a.Cin = L.cin;
+    a.Cout = L.cout;
+    a.lho = ilog2(ho);
+    a.lhin = ilog2(hi);
+    a.gather = up ? 0 : 1;
+    a.wm = g.wm[l];
+    a.wn = g.wn[l];
+    a.wblocks = a.wm * a.wn * g.chunks[l];
+    a.w = n->wbf + n->off[l];
+    a.out = l > 1 ? (void*)planes[l - 1] : (void*)n->dz[0];
+    a.oplane = pixels(l) * L.cin;
+    a.out_f32 = l == 1;
+    a.rows = up ? (int)pixels(l) : B * ho * ho;
+    const int bm = l == 3 ? 32 : 64, bn = l == 1 ? 32 : 64;  // layer 3's longest class is 64 steps: narrower tiles
+    a.xm = (a.rows + bm - 1) / bm;
+    a.xn = L.cin / bn;
+    a.xblocks = a.xm * a.xn * (up ? 1 : 4);
+    const unsigned blocks = (unsigned)(a.xblocks + a.wblocks);
+    if (l == 3)
+      grad_gemm_kernel<32, 64><<<blocks, 128, grad_smem<32, 64>(), st>>>(a);
+    else if (l == 1)
+      grad_gemm_kernel<64, 32><<<blocks, 128, grad_smem<64, 32>(), st>>>(a);
+    else
+      grad_gemm_kernel<64, 64><<<blocks, 128, grad_smem<64, 64>(), st>>>(a);
     CUDA_TRY(cudaGetLastError());
-    chunk_sum_kernel<<<(P + 255) / 256, 256, 0, st>>>(n->part, grad + n->off[l], P, wp.chunks);
-    CUDA_TRY(cudaGetLastError());
-    if (l > 0) {
-      const size_t nx = (size_t)B * Hin * Hin * L.cin;
-      conv_bwd_data_kernel<<<(int)std::min<size_t>((nx + 255) / 256, 8192), 256, 0, st>>>(
-          dz, n->wbf + n->off[l], n->act[l], n->dz[cur], B, Hin, L.cin, L.cout, L.stride, L.up, Ho);
-      CUDA_TRY(cudaGetLastError());
-      dz = n->dz[cur];
-      cur ^= 1;
-    }
   }
+  grad_first_kernel<<<g.chunks[0], 128, 0, st>>>(n->dz[0], n->act[0], n->part + g.off[0], (int)pixels(0), ilog2(h));
+  CUDA_TRY(cudaGetLastError());
+  GradSegs S{};
+  int blocks = 0;
+  auto seg = [&](int l, size_t src, int dst, int cnt) {
+    GradSeg& q = S.s[S.n++];
+    q.src = n->part + g.off[l] + src;
+    q.dst = dst;
+    q.n = cnt;
+    q.chunks = g.chunks[l];
+    q.stride = g.stride[l];
+    q.wide = q.chunks >= 16;
+    q.block0 = blocks;
+    blocks += q.wide ? (cnt + 31) / 32 : (cnt + 255) / 256;
+  };
+  for (int l = 0; l < kCnnLayers; ++l) {
+    const CnnLayer& L = kCnn[l];
+    const int nw = L.cout * 9 * L.cin;
+    seg(l, 0, n->off[l], l == 4 ? nw : nw + L.cout);
+    if (l == 4) seg(last, 18 * 64 + 2, n->off[l] + nw, L.cout);  // layer 5's blocks summed dz4
+  }
+  grad_reduce_kernel<<<blocks, 256, 0, st>>>(S, grad);
+  CUDA_TRY(cudaGetLastError());
   return MAGPIE_OK;
 }
 
@@ -2446,6 +2523,15 @@ int magpie_cnn_create(magpie_cnn** out, int32_t h, int32_t max_batch, void* stre
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(conv_fwd_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)TcConv<64>::SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(grad_gemm_kernel<64, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)grad_smem<64, 64>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(grad_gemm_kernel<32, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)grad_smem<32, 64>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(grad_gemm_kernel<64, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)grad_smem<64, 32>());
   if (e == cudaSuccess) e = cudaMemsetAsync(n->theta, 0, sizeof(float) * P, n->stream);
   if (e != cudaSuccess) {
     magpie_cnn_destroy(n);

@@ -31,7 +31,7 @@ def _stages() -> bool:
 SOURCES = [os.path.join(HERE, "csrc", f) for f in ("magpie.cu", "window_small.cu", "window_64.cu", "window_128.cu",
                                                    "window_256.cu")]
 DEPENDS = [os.path.join(HERE, "csrc", f) for f in ("core.cuh", "fft_lines.cuh", "window_kernel.cuh", "window_split.cuh", "window_body.inc",
-                                                   "window_launch.cuh", "learned.cuh", "precision.cuh", "umma.cuh",
+                                                   "window_launch.cuh", "learned.cuh", "learned_backward.cuh", "precision.cuh", "umma.cuh",
                                                    "update.cuh")]
 HEADER = os.path.join(ROOT, "include", "magpie.h")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

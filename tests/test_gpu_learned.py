@@ -336,3 +336,41 @@ def test_trained_network_effect():
           f"after 40 sweeps: objective {phi_l:.5e} vs {phi_p:.5e} plain, NRMSE {e_l:.4e} vs {e_p:.4e} plain")
     assert prop == 40 * w.n_pos and kept > 0
     assert e_l <= 1.05 * e_p and phi_l <= 1.05 * phi_p
+
+
+@pytest.mark.parametrize("h,B", [(8, 1), (8, 7), (16, 5), (32, 9), (64, 3)])
+def test_gradient_of_an_exact_forward(h, B):
+    """The backward kernels' tiles, chunks, parity classes and image edges at
+    every network side: with sparse +-1 weights and small integer inputs every
+    activation is exact in BF16, so the gradient of an arbitrary output
+    gradient has one FP64 value.  Each entry is a chain of FP32 sums (at most
+    2^15 rounded additions per layer, errors of either sign): 2e-6 of the
+    layer's norm, the bar of the test above."""
+    rng = np.random.default_rng(100 + h + B)
+    parts = []
+    for i, (ci, co) in enumerate(learned.LAYERS):
+        w = rng.choice([-1.0, 1.0], co * 9 * ci) * (rng.random(co * 9 * ci) < 1.7 / (9 * ci))
+        if i == len(learned.LAYERS) - 1:
+            w = rng.integers(-2, 3, co * 9 * ci).astype(np.float64)
+        parts += [w, rng.integers(0, 2, co).astype(np.float64)]
+    theta = np.concatenate(parts)
+    x = rng.integers(0, 3, (B, h, h, 4)).astype(np.float32)
+    yo, acts = L.forward(theta, x.astype(np.float64))
+    exact, _ = L.forward(theta, x.astype(np.float64), rounding=False)
+    assert np.array_equal(yo, exact) and all((a > 0).mean() > 0.05 for a in acts)
+    dy = rng.normal(size=(B, h, h, 2)).astype(np.float32)
+    net = net_with(theta, h, B)
+    y = torch.empty((B, h, h, 2), dtype=torch.float32, device=DEV)
+    magpie.magpie_cnn_forward(net, torch.from_numpy(x).to(DEV), y)
+    magpie.magpie_cnn_status(net)
+    assert np.array_equal(y.cpu().numpy(), yo)
+    g = torch.empty(L.param_count(), dtype=torch.float32, device=DEV)
+    magpie.magpie_cnn_backward(net, torch.from_numpy(dy).to(DEV), g)
+    gg = g.cpu().numpy().astype(np.float64)
+    go = L.backward(theta, acts, dy.astype(np.float64))
+    o = 0
+    for ci, co, _, _, _ in L.LAYERS:
+        for what, n in (("weights", co * 9 * ci), ("biases", co)):
+            # also where a batch's gradient of a layer is exactly zero
+            assert np.linalg.norm(gg[o:o + n] - go[o:o + n]) <= 2e-6 * np.linalg.norm(go[o:o + n]), (what, ci, co)
+            o += n
