@@ -37,6 +37,9 @@ struct ConvFwd {
   int B, Hin, Cin, Cout, stride, up, Ho, relu, out_f32;
   int K;       // 9 Cin
   int ksplit;  // K elements per split (multiple of 32)
+  int lho, lup;  // log2 of Ho and up
+  const float* x;  // first layer on the direct kernel: the FP32 input, rounded to BF16 into x16 as it is read
+  uint2* x16;
 };
 
 __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint32_t* b) {
@@ -215,150 +218,318 @@ __global__ void __launch_bounds__(128) conv_fwd_kernel(const ConvFwd a) {
 // and accumulate in FP32; consecutive lanes take consecutive 16-byte pieces of
 // one pixel's channels, so a warp's loads and stores are contiguous.
 //
-// Few outputs (the last layer, 64 -> 2): S = CIN / 8 lanes per output pixel,
-// lane `part` holding input channels 8 part .. 8 part + 7 of every tap; the S
-// partial sums of each output are added with butterfly shuffles.  Weights sit
-// in shared memory as BF16 [tap][co][ci], so the S lanes of a pixel read one
-// contiguous 16 S-byte row per (tap, co).  Needs `in` 16-byte aligned.
-template <int CIN, int COUT>
+// Few outputs (the last layer, 64 -> 2, input upsampled by 4): eight lanes per
+// group of four output pixels of one row, which share their input pixels
+// (three per tap row); lane `part` holds input channels 8 part .. 8 part + 7,
+// and the eight partial sums of each output are added with butterfly shuffles.
+// A tap's weights, FP32 in shared memory, are read once for the four pixels.
+// Bound by its chain of loads and shuffles; 64 windows at h = 32: 9.3 us,
+// against 20.3 with one output pixel per eight lanes, whose weights and
+// inputs were read and converted for every pixel (same sums, same order).
+// Needs `in` 16-byte aligned.
 __global__ void __launch_bounds__(256) conv_thin_out_kernel(const ConvFwd a) {
-  constexpr int S = CIN / 8;
-  static_assert(CIN % 8 == 0 && (S & (S - 1)) == 0 && S <= 32, "channel split");
-  __shared__ __align__(16) bf16 wsm[9 * COUT * CIN];
+  constexpr int CIN = 64, COUT = 2, S = CIN / 8;
+  __shared__ __align__(16) float wsm[9 * COUT * CIN];
   for (int i = threadIdx.x; i < 9 * COUT * CIN; i += blockDim.x) {
     const int co = i / (9 * CIN), r = i - co * 9 * CIN, tap = r / CIN, ci = r - tap * CIN;
-    wsm[(tap * COUT + co) * CIN + ci] = a.w[i];
+    wsm[(tap * COUT + co) * CIN + ci] = __bfloat162float(a.w[i]);
   }
+  grid_dep_wait();
+  grid_dep_launch();
   __syncthreads();
-  const int HH = a.Ho * a.Ho, Mtot = a.B * HH, Hv = a.Hin * a.up;
+  const int Hq = a.Hin, HHq = a.Ho * Hq, groups = a.B * HHq;  // groups of four pixels: Ho rows x Hin columns
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool live = t < (long long)Mtot * S;  // whole pixel groups: S divides 32
-  const int pix = live ? (int)(t / S) : 0, part = (int)(t % S);
-  const int b = pix / HH, rem = pix - b * HH, oy = rem / a.Ho, ox = rem - oy * a.Ho;
-  float acc[COUT];
+  const bool live = t < (long long)groups * S;  // whole groups: S divides 32
+  const int grp = live ? (int)(t / S) : 0, part = (int)(t % S);
+  const int b = grp / HHq, rem = grp - b * HHq, oy = rem / Hq, q = rem - oy * Hq;
+  float acc[4][COUT];
 #pragma unroll
-  for (int co = 0; co < COUT; ++co) acc[co] = 0.f;
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int co = 0; co < COUT; ++co) acc[j][co] = 0.f;
+#pragma unroll
   for (int ky = 0; ky < 3; ++ky) {
-    const int vy = oy * a.stride + ky - 1;
-    if (!live || vy < 0 || vy >= Hv) continue;
-    const bf16* rowp = a.in + (size_t)(b * a.Hin + vy / a.up) * a.Hin * CIN + part * 8;
+    const int vy = oy + ky - 1;
+    if (!live || vy < 0 || vy >= a.Ho) continue;
+    const bf16* rowp = a.in + ((size_t)(b * a.Hin + (vy >> 2)) * a.Hin + q) * CIN + part * 8;
+    float x[3][8];  // input columns q - 1, q, q + 1
+    bool ok[3];
 #pragma unroll
-    for (int kx = 0; kx < 3; ++kx) {
-      const int vx = ox * a.stride + kx - 1;
-      if (vx < 0 || vx >= Hv) continue;
-      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(rowp + (size_t)(vx / a.up) * CIN));
+    for (int e = 0; e < 3; ++e) {
+      ok[e] = e == 0 ? q > 0 : e == 2 ? q + 1 < Hq : true;
+      const uint4 raw = ok[e] ? __ldcg(reinterpret_cast<const uint4*>(rowp + (e - 1) * CIN)) : make_uint4(0, 0, 0, 0);
       const __nv_bfloat162* xh = reinterpret_cast<const __nv_bfloat162*>(&raw);
-      float x[8];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        x[2 * j] = __low2float(xh[j]);
-        x[2 * j + 1] = __high2float(xh[j]);
-      }
-#pragma unroll
-      for (int co = 0; co < COUT; ++co) {
-        const uint4 wr = *reinterpret_cast<const uint4*>(&wsm[((ky * 3 + kx) * COUT + co) * CIN + part * 8]);
-        const __nv_bfloat162* wh = reinterpret_cast<const __nv_bfloat162*>(&wr);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[co] = fmaf(x[2 * j], __low2float(wh[j]), acc[co]);
-          acc[co] = fmaf(x[2 * j + 1], __high2float(wh[j]), acc[co]);
-        }
+        x[e][2 * j] = __low2float(xh[j]);
+        x[e][2 * j + 1] = __high2float(xh[j]);
       }
     }
+#pragma unroll
+    for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+      for (int co = 0; co < COUT; ++co) {
+        const float4* wr = reinterpret_cast<const float4*>(&wsm[((ky * 3 + kx) * COUT + co) * CIN + part * 8]);
+        const float4 w0 = wr[0], w1 = wr[1];
+        const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int e = (j + kx - 1 < 0) ? 0 : (j + kx - 1 > 3) ? 2 : 1;
+          if (!ok[e]) continue;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) acc[j][co] = fmaf(x[e][c], wv[c], acc[j][co]);
+        }
+      }
   }
 #pragma unroll
-  for (int co = 0; co < COUT; ++co)
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int off = S / 2; off > 0; off >>= 1) acc[co] += __shfl_xor_sync(0xffffffffu, acc[co], off);
+    for (int co = 0; co < COUT; ++co)
+#pragma unroll
+      for (int off = S / 2; off > 0; off >>= 1) acc[j][co] += __shfl_xor_sync(0xffffffffu, acc[j][co], off);
   if (!live || part != 0) return;
+  float v[4][COUT];
 #pragma unroll
-  for (int co = 0; co < COUT; ++co) {
-    float v = acc[co] + a.bias[co];
-    if (a.relu) v = fmaxf(v, 0.f);
-    if (a.out_f32)
-      static_cast<float*>(a.out)[(size_t)pix * COUT + co] = v;
-    else
-      static_cast<bf16*>(a.out)[(size_t)pix * COUT + co] = __float2bfloat16_rn(v);
-  }
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int co = 0; co < COUT; ++co) v[j][co] = acc[j][co] + a.bias[co];
+  float4* o = reinterpret_cast<float4*>(static_cast<float*>(a.out) + ((size_t)(b * a.Ho + oy) * a.Ho + 4 * q) * COUT);
+  o[0] = make_float4(v[0][0], v[0][1], v[1][0], v[1][1]);
+  o[1] = make_float4(v[2][0], v[2][1], v[3][0], v[3][1]);
 }
 
-// Few inputs (the first layer, 4 -> 32): OS = COUT / 8 lanes per output pixel,
-// lane `part` computing outputs 8 part .. 8 part + 7 from the pixel's 9 x 4
-// inputs (one 8-byte load per tap, shared by the OS lanes).  Weights sit in
-// shared memory as FP32 [tap][ci][co]; the OS lanes of a pixel read
-// consecutive 32-byte pieces of one row.  BF16 output only, stored as one
-// 16-byte piece per lane; needs `in` 8-byte and `out` 16-byte aligned.
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) conv_thin_in_kernel(const ConvFwd a) {
-  constexpr int OS = COUT / 8;
-  static_assert(CIN == 4 && COUT % 8 == 0 && (OS & (OS - 1)) == 0 && OS <= 32, "output split");
+// Few inputs (the first layer, 4 -> 32): four lanes per group of four output
+// pixels of one row, lane `part` computing outputs 8 part .. 8 part + 7 of all
+// four from the 3 x 6 inputs around them.  A tap's weights (FP32 [tap][ci][co]
+// in shared memory) are read once for the four pixels, the FP32 input is
+// rounded to BF16 as it is read and kept for the backward pass (no conversion
+// pass).  64 windows at h = 32: 12 us, against 2.5 + 16.4 with a conversion
+// pass and one pixel per four lanes, bound by its weight reads (same sums,
+// same order).
+__global__ void __launch_bounds__(128) conv_thin_in_kernel(const ConvFwd a) {
+  constexpr int CIN = 4, COUT = 32;
   __shared__ __align__(16) float wsm[9 * CIN * COUT];
+  grid_dep_wait();
+  grid_dep_launch();
   for (int i = threadIdx.x; i < 9 * COUT * CIN; i += blockDim.x) {
     const int co = i / (9 * CIN), r = i - co * 9 * CIN;
     wsm[r * COUT + co] = __bfloat162float(a.w[i]);
   }
   __syncthreads();
-  const int HH = a.Ho * a.Ho, Mtot = a.B * HH, Hv = a.Hin * a.up;
+  const int H = a.Ho, Hg = H >> 2, groups = a.B * H * Hg;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)Mtot * OS) return;
-  const int pix = (int)(t / OS), part = (int)(t % OS);
-  const int b = pix / HH, rem = pix - b * HH, oy = rem / a.Ho, ox = rem - oy * a.Ho;
-  float acc[8];
+  if (t >= (long long)groups * 4) return;
+  const int grp = (int)(t >> 2), part = (int)(t & 3);
+  const int b = grp / (H * Hg), rem = grp - b * H * Hg, oy = rem / Hg, x0 = 4 * (rem - oy * Hg);
+  const bool vec = ((uintptr_t)a.x & 15) == 0;
+  float acc[4][8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int o = 0; o < 8; ++o) acc[j][o] = 0.f;
+#pragma unroll
   for (int ky = 0; ky < 3; ++ky) {
-    const int vy = oy * a.stride + ky - 1;
-    if (vy < 0 || vy >= Hv) continue;
-    const bf16* rowp = a.in + (size_t)(b * a.Hin + vy / a.up) * a.Hin * CIN;
+    const int iy = oy + ky - 1;
+    if (iy < 0 || iy >= H) continue;
+    const size_t row = (size_t)(b * H + iy) * H + x0;
+    float x[6][CIN];
+    bool ok[6];
 #pragma unroll
-    for (int kx = 0; kx < 3; ++kx) {
-      const int vx = ox * a.stride + kx - 1;
-      if (vx < 0 || vx >= Hv) continue;
-      const uint2 raw = __ldg(reinterpret_cast<const uint2*>(rowp + (size_t)(vx / a.up) * CIN));
-      const __nv_bfloat162* xh = reinterpret_cast<const __nv_bfloat162*>(&raw);
-      const float x[4] = {__low2float(xh[0]), __high2float(xh[0]), __low2float(xh[1]), __high2float(xh[1])};
+    for (int e = 0; e < 6; ++e) {
+      ok[e] = e == 0 ? x0 > 0 : e == 5 ? x0 + 4 < H : true;  // the middle four are the group's own
+      float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ok[e]) {
+        const float* src = a.x + (row + e - 1) * CIN;
+        f = vec ? __ldcg(reinterpret_cast<const float4*>(src))
+                : make_float4(__ldcg(src), __ldcg(src + 1), __ldcg(src + 2), __ldcg(src + 3));
+      }
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(f.x, f.y), hi = __floats2bfloat162_rn(f.z, f.w);
+      x[e][0] = __low2float(lo);
+      x[e][1] = __high2float(lo);
+      x[e][2] = __low2float(hi);
+      x[e][3] = __high2float(hi);
+      if (ky == 1 && part == 0 && e >= 1 && e <= 4)
+        a.x16[row + e - 1] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+    }
+#pragma unroll
+    for (int kx = 0; kx < 3; ++kx)
 #pragma unroll
       for (int ci = 0; ci < CIN; ++ci) {
         const float4* wr = reinterpret_cast<const float4*>(&wsm[((ky * 3 + kx) * CIN + ci) * COUT + part * 8]);
         const float4 w0 = wr[0], w1 = wr[1];
-        acc[0] = fmaf(x[ci], w0.x, acc[0]);
-        acc[1] = fmaf(x[ci], w0.y, acc[1]);
-        acc[2] = fmaf(x[ci], w0.z, acc[2]);
-        acc[3] = fmaf(x[ci], w0.w, acc[3]);
-        acc[4] = fmaf(x[ci], w1.x, acc[4]);
-        acc[5] = fmaf(x[ci], w1.y, acc[5]);
-        acc[6] = fmaf(x[ci], w1.z, acc[6]);
-        acc[7] = fmaf(x[ci], w1.w, acc[7]);
+        const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (!ok[j + kx]) continue;
+#pragma unroll
+          for (int o = 0; o < 8; ++o) acc[j][o] = fmaf(x[j + kx][ci], wv[o], acc[j][o]);
+        }
       }
-    }
   }
-  uint4 o;
-  __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    float v0 = acc[2 * j] + a.bias[part * 8 + 2 * j], v1 = acc[2 * j + 1] + a.bias[part * 8 + 2 * j + 1];
-    if (a.relu) {
-      v0 = fmaxf(v0, 0.f);
-      v1 = fmaxf(v1, 0.f);
-    }
-    oh[j] = __floats2bfloat162_rn(v0, v1);
+    uint4 o;
+    __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      oh[e] = __floats2bfloat162_rn(fmaxf(acc[j][2 * e] + a.bias[part * 8 + 2 * e], 0.f),
+                                    fmaxf(acc[j][2 * e + 1] + a.bias[part * 8 + 2 * e + 1], 0.f));
+    *reinterpret_cast<uint4*>(static_cast<bf16*>(a.out) + ((size_t)(b * H + oy) * H + x0 + j) * COUT + part * 8) = o;
   }
-  *reinterpret_cast<uint4*>(static_cast<bf16*>(a.out) + (size_t)pix * COUT + part * 8) = o;
 }
 
-// Split-K epilogue: partial sums added in split order, then bias and ReLU.
-__global__ void __launch_bounds__(256) conv_splitk_kernel(const ConvFwd a, int splits) {
-  const int Mtot = a.B * a.Ho * a.Ho;
-  const size_t n = (size_t)Mtot * a.Cout;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    float v = 0.f;
-    for (int s = 0; s < splits; ++s) v += a.part[(size_t)s * n + i];
-    v += a.bias[i % a.Cout];
-    if (a.relu) v = fmaxf(v, 0.f);
-    if (a.out_f32)
-      static_cast<float*>(a.out)[i] = v;
-    else
-      static_cast<bf16*>(a.out)[i] = __float2bfloat16_rn(v);
+// The second layer (32 -> 64, stride 2): one tap of 32 channels per step, the
+// split-K sums kept inside the block (the accumulators are added to the
+// totals where conv_fwd_kernel's splits end, so the result is bitwise its
+// split-K epilogue's).  64 pixels x 64 channels per block, four warps of
+// 32 x 32, taps brought in two steps ahead with cp.async.  64 windows at
+// h = 32: 8.7 us, against 10.3 + 6.6 with split K and its epilogue kernel.
+constexpr int kNarrowPitch = 80, kNarrowStage = 2 * 64 * kNarrowPitch;
+__global__ void __launch_bounds__(128) conv_narrow_kernel(const ConvFwd a, int lho) {
+  __shared__ __align__(16) unsigned char raw[3 * kNarrowStage];
+  const uint32_t sm = smem_addr(raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wm = warp & 1, wn = warp >> 1;
+  const int Ho = 1 << lho, Mtot = a.B << (2 * lho), bm = blockIdx.x * 64;
+  const int c = tid & 3, r0 = tid >> 2;
+  int pb[2], py[2], px[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int p = bm + r0 + 32 * i;
+    pb[i] = p < Mtot ? p >> (2 * lho) : -1;
+    py[i] = 2 * ((p >> lho) & (Ho - 1)) - 1;
+    px[i] = 2 * (p & (Ho - 1)) - 1;
+  }
+  auto copy = [](uint32_t dst, const void* src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+  };
+  auto load_w = [&](int s) {
+    const uint32_t st = sm + (uint32_t)((s % 3) * kNarrowStage + 64 * kNarrowPitch);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int n = r0 + 32 * i;
+      copy(st + (uint32_t)(n * kNarrowPitch + c * 16), a.w + (size_t)n * 288 + s * 32 + 8 * c, true);
+    }
+  };
+  auto load_a = [&](int s) {
+    const uint32_t st = sm + (uint32_t)((s % 3) * kNarrowStage);
+    const int ky = s / 3, kx = s - 3 * ky;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int iy = py[i] + ky, ix = px[i] + kx;
+      const bool ok = pb[i] >= 0 && (unsigned)iy < (unsigned)a.Hin && (unsigned)ix < (unsigned)a.Hin;
+      copy(st + (uint32_t)((r0 + 32 * i) * kNarrowPitch + c * 16),
+           a.in + (ok ? ((size_t)(pb[i] * a.Hin + iy) * a.Hin + ix) * 32 + 8 * c : 0), ok);
+    }
+  };
+  load_w(0);
+  load_w(1);
+  grid_dep_wait();
+  grid_dep_launch();
+  load_a(0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  load_a(1);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  float tot[2][4][4], acc[2][4][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) tot[i][j][e] = acc[i][j][e] = 0.f;
+  const int l7 = lane & 7, mi = lane >> 3, per = a.ksplit / 32;
+#pragma unroll 1
+  for (int s = 0; s < 9; ++s) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    if (s + 2 < 9) {
+      load_w(s + 2);
+      load_a(s + 2);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const uint32_t sa = sm + (uint32_t)((s % 3) * kNarrowStage), sb = sa + 64 * kNarrowPitch;
+#pragma unroll
+    for (int kk = 0; kk < 32; kk += 16) {
+      uint32_t af[2][4], bf[4][2];
+      auto ld4 = [](uint32_t (&r)[4], uint32_t addr) {
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(addr));
+      };
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        ld4(af[i], sa + (uint32_t)((wm * 32 + i * 16 + l7 + (mi & 1) * 8) * kNarrowPitch + (kk + (mi >> 1) * 8) * 2));
+#pragma unroll
+      for (int j = 0; j < 4; j += 2) {
+        uint32_t r[4];
+        ld4(r, sb + (uint32_t)((wn * 32 + j * 8 + (mi >> 1) * 8 + l7) * kNarrowPitch + (kk + (mi & 1) * 8) * 2));
+        bf[j][0] = r[0];
+        bf[j][1] = r[1];
+        bf[j + 1][0] = r[2];
+        bf[j + 1][1] = r[3];
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], af[i], bf[j]);
+    }
+    if ((s + 1) % per == 0 || s == 8) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            tot[i][j][e] += acc[i][j][e];
+            acc[i][j][e] = 0.f;
+          }
+    }
+  }
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const int p = bm + wm * 32 + i * 16 + g + 8 * hh;
+      if (p >= Mtot) continue;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int co = wn * 32 + j * 8 + 2 * t;
+        *reinterpret_cast<__nv_bfloat162*>(static_cast<bf16*>(a.out) + (size_t)p * 64 + co) =
+            __floats2bfloat162_rn(fmaxf(tot[i][j][2 * hh] + a.bias[co], 0.f),
+                                  fmaxf(tot[i][j][2 * hh + 1] + a.bias[co + 1], 0.f));
+      }
+    }
+}
+
+// Split-K epilogue: partial sums added in split order, then bias and ReLU;
+// four outputs per thread (Cout a power of two, n a multiple of four).
+__global__ void __launch_bounds__(256) conv_splitk_kernel(const ConvFwd a, int splits, size_t n) {
+  const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  grid_dep_wait();
+  grid_dep_launch();
+  if (i >= n) return;
+  const int c = (int)(i & (size_t)(a.Cout - 1)), cm = a.Cout - 1;
+  const float4 bi = make_float4(a.bias[c], a.bias[(c + 1) & cm], a.bias[(c + 2) & cm], a.bias[(c + 3) & cm]);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 9
+  for (int s = 0; s < splits; ++s) {
+    const float4 p = __ldcg(reinterpret_cast<const float4*>(a.part + (size_t)s * n + i));
+    v.x += p.x;
+    v.y += p.y;
+    v.z += p.z;
+    v.w += p.w;
+  }
+  v.x += bi.x;
+  v.y += bi.y;
+  v.z += bi.z;
+  v.w += bi.w;
+  if (a.relu) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+  if (a.out_f32) {
+    *reinterpret_cast<float4*>(static_cast<float*>(a.out) + i) = v;
+  } else {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(static_cast<bf16*>(a.out) + i) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
   }
 }
 
@@ -514,6 +685,82 @@ __global__ void __launch_bounds__(1024) coarse_state_kernel(const CoarseArgs A) 
   if (tid == 0) A.scale[w] = s;
 }
 
+// The same for 2 to 4 levels, whose per-pixel factors unroll (all of a coarse
+// pixel's loads in flight), on a cluster of four blocks per window: the RMS is
+// summed over the cluster.  At most four coarse pixels per thread (h <= 64).
+// Bound by the latency of its loads; m = 128, three levels, 64 windows: 12 us
+// against 18 us for the one-block form.
+template <int L>
+__global__ void __launch_bounds__(256) coarse_state_cluster_kernel(const CoarseArgs A) {
+  constexpr int F = 1 << (L - 1), NP = 4;
+  __shared__ double red[32];
+  __shared__ double share;
+  cg::cluster_group cl = cg::this_cluster();
+  const int w = blockIdx.x / 4, rank = blockIdx.x % 4, tid = threadIdx.x;
+  const int MS = A.MS, h = MS >> (L - 1), hh = h * h;
+  grid_dep_wait();
+  grid_dep_launch();
+  const int k = A.idx[w];
+  float4* xo = A.x + (size_t)w * hh;
+  if ((unsigned)k >= (unsigned)A.n_pos) {  // uniform over the cluster
+    for (int c = rank * 256 + tid; c < hh; c += 1024) xo[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (rank == 0 && tid == 0) A.scale[w] = 0.f;
+    return;
+  }
+  const int pr = A.pos[2 * k], pc = A.pos[2 * k + 1];
+  const float2* g0 = A.g0 + (size_t)w * MS * MS;
+  constexpr float norm = 1.f / (float)(F * F);
+  const float* iwH = A.pyr + lvl_off(MS, L - 1) + hh;
+  float4 v[NP];
+  float e2 = 0.f;
+#pragma unroll
+  for (int u = 0; u < NP; ++u) {
+    const int c = rank * 256 + tid + 1024 * u;
+    v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c >= hh) continue;
+    const int cy = c / h, cx = c - cy * h;
+    float2 gs = make_float2(0.f, 0.f), zs = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int fy = 0; fy < F; ++fy)
+#pragma unroll
+      for (int fx = 0; fx < F; ++fx) {
+        const int r = cy * F + fy, cc = cx * F + fx;
+        float al = norm, be = norm;
+        int woff = 0;
+#pragma unroll
+        for (int l = 0; l + 1 < L; ++l) {
+          al *= __ldg(&A.pyr[lvl_off(MS, l + 1) + (r >> (l + 1)) * (MS >> (l + 1)) + (cc >> (l + 1))]);
+          be *= __ldg(&A.wz[woff + (r >> l) * (MS >> l) + (cc >> l)]);
+          woff += (MS >> l) * (MS >> l);
+        }
+        const float2 gv = __ldcg(&g0[r * MS + cc]);
+        const float2 zv = __ldcg(&A.z[(size_t)(pr + r) * A.n_cols + pc + cc]);
+        gs.x = fmaf(al, gv.x, gs.x);
+        gs.y = fmaf(al, gv.y, gs.y);
+        zs.x = fmaf(be, zv.x, zs.x);
+        zs.y = fmaf(be, zv.y, zs.y);
+      }
+    const float iw = __ldg(&iwH[c]);
+    v[u] = make_float4(zs.x, zs.y, gs.x * iw, gs.y * iw);
+    e2 += v[u].z * v[u].z + v[u].w * v[u].w;
+  }
+  const double part = block_sum((double)e2, red, tid, 256);  // valid in thread 0
+  if (tid == 0) share = part;
+  cl.sync();
+  double tot = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) tot += *cl.map_shared_rank(&share, q);
+  const float s = (float)sqrt(tot / (double)hh);
+  const float is = s > 1e-30f ? 1.f / s : 0.f;
+#pragma unroll
+  for (int u = 0; u < NP; ++u) {
+    const int c = rank * 256 + tid + 1024 * u;
+    if (c < hh) xo[c] = make_float4(v[u].x, v[u].y, v[u].z * is, v[u].w * is);
+  }
+  if (rank == 0 && tid == 0) A.scale[w] = s;
+  cl.sync();  // no block leaves while another may still read its share
+}
+
 struct LearnedUpArgs {
   const int32_t* idx;  // [count]
   int n_pos, MS, L;
@@ -533,39 +780,67 @@ __host__ __device__ __forceinline__ int up_off(int MS, int l) {
   return o;
 }
 
-// One block per window: the V-cycle above the finest level in residual form,
-// from g^0 in the increments, in shared memory.  LEARN: two float2 pyramids of
-// levels 1 .. L-1 (plain and learned coarsest correction), the surrogate test
-// and the kept one written back as w^0 Delta; otherwise one pyramid (the plain
-// MAGPS V-cycle, as the window kernel's pass D computes it).
-template <bool LEARN>
-__global__ void __launch_bounds__(1024) vcycle_up_kernel(const LearnedUpArgs A) {
+// The V-cycle above the finest level in residual form, from g^0 in the
+// increments, with the plain and the learned coarsest correction side by side;
+// the surrogate test keeps one of them, written back as w^0 Delta.  A cluster
+// of kUpSplit blocks per window, each with 1 / kUpSplit of the rows (whole
+// coarsest bins: the network's side h is a multiple of 8): only the surrogate
+// difference crosses blocks.  A thread keeps the g^0 of its 2 x 2 bins in
+// registers from the restriction to the write-back, so g^0 is read once.
+// Shared memory: two float2 pyramids of this block's rows of levels 1 .. L-1.
+// m = 128, three levels, 64 windows: 12.7 us, against 26 with one block of
+// 1024 threads per window that read g^0 three times.
+constexpr int kUpSplit = 8, kUpThreads = 256;
+__global__ void __launch_bounds__(kUpThreads) vcycle_up_kernel(const LearnedUpArgs A) {
   extern __shared__ __align__(16) unsigned char lsm[];
   __shared__ double red[32];
-  __shared__ int keep;
-  const int w = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+  __shared__ double share;
+  cg::cluster_group cl = cg::this_cluster();
+  constexpr int nt = kUpThreads, NB = 2;  // bins per thread: (MS / 2)^2 / 8 <= 512
+  const int w = blockIdx.x / kUpSplit, q = blockIdx.x % kUpSplit, tid = threadIdx.x;
   const int MS = A.MS, L = A.L, M = MS * MS;
+  grid_dep_wait();
+  grid_dep_launch();
   const int k = A.idx[w];
-  if ((unsigned)k >= (unsigned)A.n_pos) {
-    if (LEARN && tid == 0) {
+  if ((unsigned)k >= (unsigned)A.n_pos) {  // uniform over the cluster
+    if (q == 0 && tid == 0) {
       A.accepted[w] = 0;
       A.margin[w] = 0.0;
     }
     return;
   }
-  const int tot = up_off(MS, L);
+  const int tot = up_off(MS, L) / kUpSplit;
   float2* Ep = reinterpret_cast<float2*>(lsm);
-  float2* En = LEARN ? Ep + tot : Ep;
+  float2* En = Ep + tot;
   float2* g0 = A.contrib + (size_t)w * M;
+  // level l: this block's rows q n / 8 .. of n = MS >> l, at up_off / 8
+  const auto off = [&](int l) { return up_off(MS, l) / kUpSplit; };
 
   // ---- g^l, l = 1 .. L-1: g^{l+1} = W_u^l . I(g^l)
-  for (int l = 1; l < L; ++l) {
-    const int s = MS >> l, sf = MS >> (l - 1);
-    const float* wu = A.pyr + lvl_off(MS, l);
-    float2* dst = Ep + up_off(MS, l);
-    const float2* src = (l == 1) ? g0 : Ep + up_off(MS, l - 1);
-    for (int i = tid; i < s * s; i += nt) {
-      const int r = i / s, c = i - r * s;
+  float4 gr[NB][2];  // the two rows of each of this thread's finest bins
+  const int s1 = MS >> 1, nb = s1 * s1 / kUpSplit, ls1 = 31 - __clz(s1);
+  {
+    const float* wu = A.pyr + lvl_off(MS, 1) + q * nb;
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int i = tid + nt * u;
+      if (i >= nb) continue;
+      const int r = (q * nb + i) >> ls1, c = i & (s1 - 1);
+      gr[u][0] = __ldcg(reinterpret_cast<const float4*>(&g0[(2 * r) * MS + 2 * c]));
+      gr[u][1] = __ldcg(reinterpret_cast<const float4*>(&g0[(2 * r + 1) * MS + 2 * c]));
+      const float f = 0.25f * __ldg(&wu[i]);
+      Ep[i] = make_float2(f * (gr[u][0].x + gr[u][0].z + gr[u][1].x + gr[u][1].z),
+                          f * (gr[u][0].y + gr[u][0].w + gr[u][1].y + gr[u][1].w));
+    }
+    __syncthreads();
+  }
+  for (int l = 2; l < L; ++l) {
+    const int s = MS >> l, sf = MS >> (l - 1), n = s * s / kUpSplit, ls = 31 - __clz(s);
+    const float* wu = A.pyr + lvl_off(MS, l) + q * n;
+    float2* dst = Ep + off(l);
+    const float2* src = Ep + off(l - 1);
+    for (int i = tid; i < n; i += nt) {
+      const int r = i >> ls, c = i & (s - 1);
       const float2 a = src[(2 * r) * sf + 2 * c], b = src[(2 * r) * sf + 2 * c + 1];
       const float2 cc = src[(2 * r + 1) * sf + 2 * c], d = src[(2 * r + 1) * sf + 2 * c + 1];
       const float f = 0.25f * __ldg(&wu[i]);
@@ -574,92 +849,107 @@ __global__ void __launch_bounds__(1024) vcycle_up_kernel(const LearnedUpArgs A) 
     __syncthreads();
   }
   // ---- coarsest: plain step and proposal
-  const float s = LEARN ? A.scale[w] : 0.f;
-  const bool proposed = LEARN && s > 1e-30f;
+  const float s = A.scale[w];
+  const bool proposed = s > 1e-30f;
   {
-    const int h = MS >> (L - 1);
-    const float* iw = A.pyr + lvl_off(MS, L - 1) + h * h;
-    float2* P = Ep + up_off(MS, L - 1);
-    float2* N = En + up_off(MS, L - 1);
-    const float2* yy = LEARN ? reinterpret_cast<const float2*>(A.y) + (size_t)w * h * h : nullptr;
-    for (int i = tid; i < h * h; i += nt) {
+    const int h = MS >> (L - 1), n = h * h / kUpSplit;
+    const float* iw = A.pyr + lvl_off(MS, L - 1) + h * h + q * n;
+    float2* P = Ep + off(L - 1);
+    float2* N = En + off(L - 1);
+    const float2* yy = reinterpret_cast<const float2*>(A.y) + (size_t)w * h * h + q * n;
+    for (int i = tid; i < n; i += nt) {
       const float2 g = P[i];
       const float f = __ldg(&iw[i]);
       const float2 e = make_float2(g.x * f, g.y * f);
       P[i] = e;
-      if (LEARN) {
-        if (proposed) {
-          const float2 d = yy[i];
-          N[i] = make_float2(e.x + s * d.x, e.y + s * d.y);
-        } else {
-          N[i] = e;
-        }
+      if (proposed) {
+        const float2 d = __ldcg(&yy[i]);
+        N[i] = make_float2(e.x + s * d.x, e.y + s * d.y);
+      } else {
+        N[i] = e;
       }
     }
   }
   __syncthreads();
   // ---- up: e^l = g^l / w^l + (u^l / w^l) I_H^h e^{l+1}, l = L-2 .. 1
   for (int l = L - 2; l >= 1; --l) {
-    const int s2 = MS >> l, sc = MS >> (l + 1);
-    const float* iw = A.pyr + lvl_off(MS, l) + s2 * s2;
+    const int s2 = MS >> l, sc = MS >> (l + 1), n = s2 * s2 / kUpSplit, ls = 31 - __clz(s2);
+    const float* iw = A.pyr + lvl_off(MS, l) + s2 * s2 + q * n;
     const float* rr = iw + s2 * s2;
-    float2* P = Ep + up_off(MS, l);
-    float2* N = En + up_off(MS, l);
-    const float2* Pc = Ep + up_off(MS, l + 1);
-    const float2* Nc = En + up_off(MS, l + 1);
-    for (int i = tid; i < s2 * s2; i += nt) {
-      const int r = i / s2, c = i - r * s2;
-      const int pi = (r >> 1) * sc + (c >> 1);
+    float2* P = Ep + off(l);
+    float2* N = En + off(l);
+    const float2* Pc = Ep + off(l + 1);
+    const float2* Nc = En + off(l + 1);
+    for (int i = tid; i < n; i += nt) {
+      const int pi = (i >> (ls + 1)) * sc + ((i & (s2 - 1)) >> 1);
       const float2 g = P[i];
-      const float f = __ldg(&iw[i]), q = __ldg(&rr[i]);
-      const float2 ep = Pc[pi];
-      if (LEARN) {
-        const float2 en = Nc[pi];
-        N[i] = make_float2(g.x * f + q * en.x, g.y * f + q * en.y);
-      }
-      P[i] = make_float2(g.x * f + q * ep.x, g.y * f + q * ep.y);
+      const float f = __ldg(&iw[i]), qq = __ldg(&rr[i]);
+      const float2 ep = Pc[pi], en = Nc[pi];
+      N[i] = make_float2(g.x * f + qq * en.x, g.y * f + qq * en.y);
+      P[i] = make_float2(g.x * f + qq * ep.x, g.y * f + qq * ep.y);
     }
     __syncthreads();
   }
+  // ---- finest: w^0 Delta = g^0 + u^0 I_H^h e^1; surrogate difference
+  // 1/2 |Q|^2 |Delta|^2 - Re(conj(Delta) g^0) summed for both candidates
   const float* u0 = A.pyr;
   const float* w0 = A.pyr + M;
-  const int s1 = MS >> 1;
-  if (LEARN) {
-    // ---- finest: w^0 Delta = g^0 + u^0 I_H^h e^1; surrogate difference
-    // 1/2 |Q|^2 |Delta|^2 - Re(conj(Delta) g^0) summed for both candidates
-    float dsum = 0.f;
-    for (int i = tid; i < M; i += nt) {
-      const int r = i / MS, c = i - r * MS;
-      const int pi = (r >> 1) * s1 + (c >> 1);
-      const float2 g = g0[i];
-      const float u = __ldg(&u0[i]), wv = __ldg(&w0[i]);
-      const float iwv = wv > 1e-30f ? 1.f / wv : 0.f;
-      const float q2 = wv - u;
-      const float2 ep = Ep[pi], en = En[pi];
-      const float2 dp = make_float2((g.x + u * ep.x) * iwv, (g.y + u * ep.y) * iwv);
-      const float2 dn = make_float2((g.x + u * en.x) * iwv, (g.y + u * en.y) * iwv);
-      const float sp = 0.5f * q2 * (dp.x * dp.x + dp.y * dp.y) - (dp.x * g.x + dp.y * g.y);
-      const float sn = 0.5f * q2 * (dn.x * dn.x + dn.y * dn.y) - (dn.x * g.x + dn.y * g.y);
-      dsum += sp - sn;
+  float2 uu[NB][2];
+  float dsum = 0.f;
+#pragma unroll
+  for (int u = 0; u < NB; ++u) {
+    const int i = tid + nt * u;
+    if (i >= nb) continue;
+    const int r = (q * nb + i) >> ls1, c = i & (s1 - 1);
+    const float2 ep = Ep[i], en = En[i];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const int o = (2 * r + a) * MS + 2 * c;
+      uu[u][a] = __ldg(reinterpret_cast<const float2*>(&u0[o]));
+      const float2 wv2 = __ldg(reinterpret_cast<const float2*>(&w0[o]));
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const float2 g = b ? make_float2(gr[u][a].z, gr[u][a].w) : make_float2(gr[u][a].x, gr[u][a].y);
+        const float uv = b ? uu[u][a].y : uu[u][a].x, wv = b ? wv2.y : wv2.x;
+        const float iwv = wv > 1e-30f ? 1.f / wv : 0.f;
+        const float q2 = wv - uv;
+        const float2 dp = make_float2((g.x + uv * ep.x) * iwv, (g.y + uv * ep.y) * iwv);
+        const float2 dn = make_float2((g.x + uv * en.x) * iwv, (g.y + uv * en.y) * iwv);
+        const float sp = 0.5f * q2 * (dp.x * dp.x + dp.y * dp.y) - (dp.x * g.x + dp.y * g.y);
+        const float sn = 0.5f * q2 * (dn.x * dn.x + dn.y * dn.y) - (dn.x * g.x + dn.y * g.y);
+        dsum += sp - sn;
+      }
     }
-    const double mg = block_sum((double)dsum, red, tid, nt);
-    if (tid == 0) {
-      keep = (proposed && mg >= 0.0) ? 1 : 0;
-      A.accepted[w] = keep;
-      A.margin[w] = proposed ? mg : 0.0;
-      if (proposed) atomicAdd(&A.stats[0], 1ull);
-      if (keep) atomicAdd(&A.stats[1], 1ull);
+  }
+  const double part = block_sum((double)dsum, red, tid, nt);  // valid in thread 0
+  if (tid == 0) share = part;
+  cl.sync();
+  double mg = 0.0;
+#pragma unroll
+  for (int j = 0; j < kUpSplit; ++j) mg += *cl.map_shared_rank(&share, j);
+  const bool keep = proposed && mg >= 0.0;
+  if (q == 0 && tid == 0) {
+    A.accepted[w] = keep;
+    A.margin[w] = proposed ? mg : 0.0;
+    if (proposed) atomicAdd(&A.stats[0], 1ull);
+    if (keep) atomicAdd(&A.stats[1], 1ull);
+  }
+  const float2* E = keep ? En : Ep;
+#pragma unroll
+  for (int u = 0; u < NB; ++u) {
+    const int i = tid + nt * u;
+    if (i >= nb) continue;
+    const int r = (q * nb + i) >> ls1, c = i & (s1 - 1);
+    const float2 e = E[i];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const float2 uv = uu[u][a];
+      const float4 g = gr[u][a];
+      *reinterpret_cast<float4*>(&g0[(2 * r + a) * MS + 2 * c]) =
+          make_float4(g.x + uv.x * e.x, g.y + uv.x * e.y, g.z + uv.y * e.x, g.w + uv.y * e.y);
     }
-    __syncthreads();
   }
-  const float2* E = (LEARN && keep) ? En : Ep;
-  for (int i = tid; i < M; i += nt) {
-    const int r = i / MS, c = i - r * MS;
-    const float2 e = E[(r >> 1) * s1 + (c >> 1)];
-    const float u = __ldg(&u0[i]);
-    const float2 g = g0[i];
-    g0[i] = make_float2(g.x + u * e.x, g.y + u * e.y);
-  }
+  cl.sync();  // no block leaves while another may still read its share
 }
 
 // patches[w] = the m x m window of the object at window idx[w] (zeros for an

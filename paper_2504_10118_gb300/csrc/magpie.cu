@@ -572,12 +572,6 @@ cudaError_t prepare_kernels(int MS) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(apply_kernel_batched<32, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(sizeof(ApplyEntry) * kMaxMinibatch));
-  if (e == cudaSuccess && MS <= 128)
-    e = cudaFuncSetAttribute(vcycle_up_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(2 * sizeof(float2) * (size_t)up_off(128, 8)));
-  if (e == cudaSuccess && MS >= 64)
-    e = cudaFuncSetAttribute(vcycle_up_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(float2) * (size_t)up_off(MS, ilog2(MS) + 1)));
   if (e != cudaSuccess) return e;
   switch (MS) {
 #define MAGPIE_CASE(S) \
@@ -876,13 +870,13 @@ ConvPlan conv_plan(const ConvFwd& a) {
 // tap (Cin a multiple of 64) and whole 64-wide N tiles.
 bool conv_tc_fits(const ConvFwd& a) { return a.Cin % 64 == 0 && a.Cout % 64 == 0; }
 // Thin layers the direct FP32-FMA kernels serve: the network's first (4 -> 32,
-// BF16 output) and last (64 -> 2) convolutions, with the alignment their
-// 16-byte (8-byte) loads and stores need.
+// from the FP32 input) and last (64 -> 2, input upsampled by 4) convolutions.
 bool conv_direct_fits(const ConvFwd& a) {
-  const auto al = [](const void* p, uintptr_t n) { return ((uintptr_t)p & (n - 1)) == 0; };
-  if (a.Cin == 64 && a.Cout == 2) return al(a.in, 16);
-  if (a.Cin == 4 && a.Cout == 32) return !a.out_f32 && al(a.in, 8) && al(a.out, 16);
-  return false;
+  return (a.Cin == 64 && a.Cout == 2 && a.up == 4 && a.stride == 1 && a.out_f32) || (a.Cin == 4 && a.Cout == 32 && a.x);
+}
+// The network's second convolution.
+bool conv_narrow_fits(const ConvFwd& a) {
+  return a.Cin == 32 && a.Cout == 64 && a.stride == 2 && a.up == 1 && a.relu && !a.out_f32;
 }
 
 // Tiles of the tcgen05 convolution: 128 output pixels x 128 (or 64) output
@@ -972,38 +966,40 @@ cudaError_t launch_conv(const ConvFwd& a0, float* part, cudaStream_t st, int ten
   a.ksplit = pl.ksplit;
   a.part = pl.splits > 1 ? part : nullptr;
   const dim3 grid(pl.gx, pl.gy, pl.splits);
+  // path 1: each kernel a programmatic dependent of the one before
   if (tensor_path == 1 && conv_direct_fits(a)) {
-    const long long pixels = (long long)a.B * a.Ho * a.Ho;
-    if (a.Cin == 64) {  // 8 lanes per pixel
-      conv_thin_out_kernel<64, 2><<<(int)((pixels * 8 + 255) / 256), 256, 0, st>>>(a);
-    } else {  // 4 lanes per pixel
-      conv_thin_in_kernel<4, 32><<<(int)((pixels * 4 + 255) / 256), 256, 0, st>>>(a);
-    }
-    return cudaGetLastError();
+    const long long groups = (long long)a.B * a.Ho * (a.Ho / 4);  // of four pixels
+    if (a.Cin == 64)  // 8 lanes per group
+      return launch_ex(conv_thin_out_kernel, dim3((unsigned)((groups * 8 + 255) / 256)), dim3(256), 0, st, 1, true, a);
+    return launch_ex(conv_thin_in_kernel, dim3((unsigned)((groups * 4 + 127) / 128)), dim3(128), 0, st, 1, true, a);
   }
+  if (tensor_path == 1 && conv_narrow_fits(a))
+    return launch_ex(conv_narrow_kernel, dim3((unsigned)((a.B * a.Ho * a.Ho + 63) / 64)), dim3(128), 0, st, 1, true, a,
+                     a.lho);
+  cudaError_t e;
   if (tc && pl.bn == 128)
-    conv_fwd_tc_kernel<128><<<grid, 128, TcConv<128>::SMEM, st>>>(a, err);
+    e = launch_ex(conv_fwd_tc_kernel<128>, grid, dim3(128), TcConv<128>::SMEM, st, 1, true, a, err);
   else if (tc)
-    conv_fwd_tc_kernel<64><<<grid, 128, TcConv<64>::SMEM, st>>>(a, err);
+    e = launch_ex(conv_fwd_tc_kernel<64>, grid, dim3(128), TcConv<64>::SMEM, st, 1, true, a, err);
   else if (pl.bn == 8)
-    conv_fwd_kernel<128, 8><<<grid, 128, 0, st>>>(a);
+    e = launch_ex(conv_fwd_kernel<128, 8>, grid, dim3(128), 0, st, 1, false, a);
   else if (pl.bn == 32)
-    conv_fwd_kernel<128, 32><<<grid, 128, 0, st>>>(a);
+    e = launch_ex(conv_fwd_kernel<128, 32>, grid, dim3(128), 0, st, 1, false, a);
   else
-    conv_fwd_kernel<64, 64><<<grid, 128, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
+    e = launch_ex(conv_fwd_kernel<64, 64>, grid, dim3(128), 0, st, 1, false, a);
   if (e != cudaSuccess || pl.splits == 1) return e;
   const size_t n = (size_t)a.B * a.Ho * a.Ho * a.Cout;
-  conv_splitk_kernel<<<(int)std::min<size_t>((n + 255) / 256, 4096), 256, 0, st>>>(a, pl.splits);
-  return cudaGetLastError();
+  return launch_ex(conv_splitk_kernel, dim3((unsigned)((n / 4 + 255) / 256)), dim3(256), 0, st, 1, tc, a, pl.splits, n);
 }
 
 // Forward pass of `batch` inputs x [batch][h][h][4] (float) into y [batch][h][h][2].
 int cnn_enqueue_forward(magpie_cnn* n, const float* x, int batch, float* y, cudaStream_t st) {
   const int h = n->h;
-  const size_t nx = (size_t)batch * h * h * 4;
-  to_bf16_kernel<<<(int)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, st>>>(x, n->act[0], nx);
-  CUDA_TRY(cudaGetLastError());
+  if (n->tensor_path == 0) {  // the first layer of path 1 rounds the input as it reads it
+    const size_t nx = (size_t)batch * h * h * 4;
+    to_bf16_kernel<<<(int)std::min<size_t>((nx + 255) / 256, 4096), 256, 0, st>>>(x, n->act[0], nx);
+    CUDA_TRY(cudaGetLastError());
+  }
   for (int l = 0; l < kCnnLayers; ++l) {
     const CnnLayer& L = kCnn[l];
     ConvFwd a{};
@@ -1021,6 +1017,12 @@ int cnn_enqueue_forward(magpie_cnn* n, const float* x, int batch, float* y, cuda
     a.relu = L.relu;
     a.out_f32 = l + 1 == kCnnLayers;
     a.K = 9 * L.cin;
+    a.lho = ilog2(a.Ho);
+    a.lup = ilog2(L.up);
+    if (l == 0 && n->tensor_path == 1) {
+      a.x = x;
+      a.x16 = reinterpret_cast<uint2*>(n->act[0]);
+    }
     CUDA_TRY(launch_conv(a, n->part, st, n->tensor_path, n->err));
   }
   n->last_batch = batch;
@@ -1168,7 +1170,19 @@ CoarseArgs coarse_args(magpie_ctx* c, const int32_t* idx, float4* x, float* scal
   return a;
 }
 
-size_t learned_up_smem(int MS, int L) { return 2 * sizeof(float2) * (size_t)up_off(MS, L); }
+cudaError_t launch_coarse_state(const CoarseArgs& a, int count, cudaStream_t st) {
+  // the cluster kernels store whole float4 (a caller's x may be less aligned) and
+  // keep at most four coarse pixels per thread
+  const bool fits = ((uintptr_t)a.x & 15) == 0 && (a.MS >> (a.L - 1)) <= 64;
+  const dim3 grid(4 * (unsigned)count), block(256);
+  if (fits && a.L == 2) return launch_ex(coarse_state_cluster_kernel<2>, grid, block, 0, st, 4, true, a);
+  if (fits && a.L == 3) return launch_ex(coarse_state_cluster_kernel<3>, grid, block, 0, st, 4, true, a);
+  if (fits && a.L == 4) return launch_ex(coarse_state_cluster_kernel<4>, grid, block, 0, st, 4, true, a);
+  return launch_ex(coarse_state_kernel, dim3((unsigned)count), dim3(1024), 0, st, 1, false, a);
+}
+
+// dynamic shared memory of vcycle_up_kernel (two pyramids of an eighth of the window)
+size_t learned_up_smem(int MS, int L) { return 2 * sizeof(float2) * (size_t)(up_off(MS, L) / kUpSplit); }
 
 LearnedUpArgs up_args(magpie_ctx* c, const int32_t* idx) {
   LearnedUpArgs u{};
@@ -1185,8 +1199,7 @@ LearnedUpArgs up_args(magpie_ctx* c, const int32_t* idx) {
 // pass, then the V-cycle with the kept coarse correction writes w^0 Delta
 // back to the increments.
 int enqueue_learned_tail(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st) {
-  coarse_state_kernel<<<count, 1024, 0, st>>>(coarse_args(c, idx, c->lx, c->lscale));
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(launch_coarse_state(coarse_args(c, idx, c->lx, c->lscale), count, st));
   int rc = cnn_enqueue_forward(c->cnn, reinterpret_cast<const float*>(c->lx), count, c->cnn->y, st);
   if (rc) return rc;
   LearnedUpArgs u = up_args(c, idx);
@@ -1195,8 +1208,8 @@ int enqueue_learned_tail(magpie_ctx* c, const int32_t* idx, int count, cudaStrea
   u.accepted = c->lacc;
   u.margin = c->lmargin;
   u.stats = c->lstats;
-  vcycle_up_kernel<true><<<count, 1024, learned_up_smem(c->p.m, c->p.levels), st>>>(u);
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(launch_ex(vcycle_up_kernel, dim3(kUpSplit * (unsigned)count), dim3(kUpThreads),
+                     learned_up_smem(c->p.m, c->p.levels), st, kUpSplit, true, u));
   return MAGPIE_OK;
 }
 
@@ -2604,8 +2617,7 @@ int magpie_coarse_state(magpie_ctx* c, const int32_t* idx, int32_t count, float*
   StepArgs a = make_args(c, idx);
   a.grad_only = 1;
   CUDA_TRY(launch_window_m<kStep>(c->p.m, a, count, c->stream));
-  coarse_state_kernel<<<count, 1024, 0, c->stream>>>(coarse_args(c, idx, reinterpret_cast<float4*>(x), scale));
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(launch_coarse_state(coarse_args(c, idx, reinterpret_cast<float4*>(x), scale), count, c->stream));
   return read_err(c);
 }
 
