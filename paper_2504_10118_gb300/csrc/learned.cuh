@@ -721,25 +721,39 @@ __global__ void __launch_bounds__(256) coarse_state_cluster_kernel(const CoarseA
     const int cy = c / h, cx = c - cy * h;
     float2 gs = make_float2(0.f, 0.f), zs = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int fy = 0; fy < F; ++fy)
+    for (int fy = 0; fy < F; ++fy) {
+      const int r = cy * F + fy;
+      // two pixels at a time: g^0 and W_z^0 by aligned 16- and 8-byte loads
 #pragma unroll
-      for (int fx = 0; fx < F; ++fx) {
-        const int r = cy * F + fy, cc = cx * F + fx;
-        float al = norm, be = norm;
-        int woff = 0;
+      for (int fx = 0; fx < F; fx += 2) {
+        const int cc = cx * F + fx;
+        float al = norm;  // shared by both pixels
 #pragma unroll
-        for (int l = 0; l + 1 < L; ++l) {
+        for (int l = 0; l + 1 < L; ++l)
           al *= __ldg(&A.pyr[lvl_off(MS, l + 1) + (r >> (l + 1)) * (MS >> (l + 1)) + (cc >> (l + 1))]);
-          be *= __ldg(&A.wz[woff + (r >> l) * (MS >> l) + (cc >> l)]);
+        const float2 w0 = __ldg(reinterpret_cast<const float2*>(&A.wz[r * MS + cc]));
+        const float4 gv = __ldcg(reinterpret_cast<const float4*>(&g0[r * MS + cc]));
+        const float2* zp = &A.z[(size_t)(pr + r) * A.n_cols + pc + cc];
+        const float2 z0 = __ldcg(zp), z1 = __ldcg(zp + 1);
+        float be0 = norm * w0.x, be1 = norm * w0.y;
+        int woff = MS * MS;
+#pragma unroll
+        for (int l = 1; l + 1 < L; ++l) {
+          const float b2 = __ldg(&A.wz[woff + (r >> l) * (MS >> l) + (cc >> l)]);
+          be0 *= b2;
+          be1 *= b2;
           woff += (MS >> l) * (MS >> l);
         }
-        const float2 gv = __ldcg(&g0[r * MS + cc]);
-        const float2 zv = __ldcg(&A.z[(size_t)(pr + r) * A.n_cols + pc + cc]);
         gs.x = fmaf(al, gv.x, gs.x);
         gs.y = fmaf(al, gv.y, gs.y);
-        zs.x = fmaf(be, zv.x, zs.x);
-        zs.y = fmaf(be, zv.y, zs.y);
+        zs.x = fmaf(be0, z0.x, zs.x);
+        zs.y = fmaf(be0, z0.y, zs.y);
+        gs.x = fmaf(al, gv.z, gs.x);
+        gs.y = fmaf(al, gv.w, gs.y);
+        zs.x = fmaf(be1, z1.x, zs.x);
+        zs.y = fmaf(be1, z1.y, zs.y);
       }
+    }
     const float iw = __ldg(&iwH[c]);
     v[u] = make_float4(zs.x, zs.y, gs.x * iw, gs.y * iw);
     e2 += v[u].z * v[u].z + v[u].w * v[u].w;
