@@ -68,6 +68,9 @@ cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
 // the window kernel in mode `mode` (a Mode) over `windows` windows;
 template <int MS>
 cudaError_t window_launch(int mode, const StepArgs& a, int windows, cudaStream_t st);
+// forward intensities of windows 0 .. windows - 1 (tw: MS twiddles, host);
+template <int MS>
+cudaError_t window_sim_launch(const StepArgs& a, const float2* tw, int windows, cudaStream_t st);
 // the batched minibatch-step kernel with register bound `minb` (blocks per SM);
 template <int MS>
 cudaError_t window_launch_batched(const StepArgs* table, const int2* map, int windows, cudaStream_t st, int minb);

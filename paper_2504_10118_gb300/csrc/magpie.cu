@@ -525,6 +525,17 @@ cudaError_t launch_window_batched_m(int MS, const StepArgs* table, const int2* m
   }
 }
 
+cudaError_t launch_sim_m(int MS, const StepArgs& a, const float2* tw, int windows, cudaStream_t st) {
+  switch (MS) {
+#define MAGPIE_CASE(S) \
+  case S:              \
+    return window_sim_launch<S>(a, tw, windows, st);
+    MAGPIE_WINDOW_SIZES(MAGPIE_CASE)
+#undef MAGPIE_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 // The split form's kernels for window side MS (64 and more).
 cudaError_t split_launch_m(int MS, bool atomic, bool early, const StepArgs& a, int windows, cudaStream_t st) {
   switch (MS) {
@@ -2177,15 +2188,6 @@ int magpie_forward_intensities(const void* object, int32_t n_rows, int32_t n_col
   CUDA_TRY(cudaStreamSynchronize(st));
   rc = check_positions(hpos.data(), n_pos, n_rows, n_cols, m);
   if (rc) return rc;
-  CUDA_TRY(prepare_kernels(m));
-  float2* tw = nullptr;
-  int32_t* iota = nullptr;
-  CUDA_TRY(cudaMalloc((void**)&tw, sizeof(float2) * m));
-  cudaError_t e = cudaMalloc((void**)&iota, sizeof(int32_t) * n_pos);
-  if (e != cudaSuccess) {
-    cudaFree(tw);
-    CUDA_TRY(e);
-  }
   std::vector<float2> htw(m);
   for (int t = 0; t < m; ++t) {
     const double ang = -2.0 * 3.14159265358979323846 * (double)t / (double)m;
@@ -2196,22 +2198,12 @@ int magpie_forward_intensities(const void* object, int32_t n_rows, int32_t n_col
   a.n_rows = n_rows;
   a.n_cols = n_cols;
   a.Q = (const float2*)probe;
-  a.tw = tw;
   a.out_int = out;
   a.pos = positions;
-  a.idx = iota;
   a.n_pos = n_pos;
   a.levels = 1;
-  e = cudaMemcpyAsync(tw, htw.data(), sizeof(float2) * m, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) {
-    iota_kernel<<<(n_pos + 255) / 256, 256, 0, st>>>(iota, n_pos);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = launch_window_m<kSim>(m, a, n_pos, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(tw);
-  cudaFree(iota);
-  CUDA_TRY(e);
+  CUDA_TRY(launch_sim_m(m, a, htw.data(), n_pos, st));
+  CUDA_TRY(cudaStreamSynchronize(st));
   return MAGPIE_OK;
 }
 
