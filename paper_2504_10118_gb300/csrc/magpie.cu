@@ -773,7 +773,7 @@ struct magpie_ctx {
   float2* g1buf = nullptr;    // [minibatch][m/2][m/2] level-1 residual gradient, then increment
   float2* g2buf = nullptr;    // [minibatch][m/4][m/4] level-2 residual gradient (three levels or more)
   int* hand = nullptr;        // [3][minibatch] window hand-off counts of the transform kernels
-  TcTables* tabs = nullptr;
+  TcTables* tabs[2] = {nullptr, nullptr};  // of the register-fragment and the tcgen05 path
   cudaGraphExec_t graph = nullptr;
   // pipelined host sweeps (magpie_sweep_host_async): two amplitude buffers,
   // their raw-intensity staging, a sweep graph per buffer, and per buffer the
@@ -1225,30 +1225,74 @@ int enqueue_learned_tail(magpie_ctx* c, const int32_t* idx, int count, cudaStrea
 }
 
 // ----------------------------------------------------------- precision form
-void build_tc_tables(int MS, TcTables& T) {
-  const int QR = MS / 16;
+// The tables of one MMA path (0: register fragments, 1: tcgen05).
+void build_tc_tables(int MS, int path, TcTables& T) {
+  const int QR = MS / 16, K2T = (2 * QR + 15) / 16, N2T = 2 * QR / 8, Q2 = 2 * QR < 16 ? 16 : 2 * QR;
   const double pi = 3.14159265358979323846;
   std::memset(&T, 0, sizeof(T));
+  const auto half_bits = [](__half h) {
+    uint16_t b;
+    std::memcpy(&b, &h, sizeof(b));
+    return (uint32_t)b;
+  };
+  // hi (part 0) or lo (part 1) FP16 of two consecutive values
+  const auto pair = [&](float a, float b, int part) {
+    const __half ha = __float2half_rn(a), hb = __float2half_rn(b);
+    if (!part) return half_bits(ha) | (half_bits(hb) << 16);
+    return half_bits(__float2half_rn(a - __half2float(ha))) | (half_bits(__float2half_rn(b - __half2float(hb))) << 16);
+  };
   for (int inv = 0; inv < 2; ++inv) {
+    float f16[32][32] = {}, fq[32][32] = {};
     const double sg = inv ? 1.0 : -1.0;
     for (int k = 0; k < 16; ++k)
       for (int n = 0; n < 16; ++n) {
         const double ph = 2.0 * pi * (double)((k * n) % 16) / 16.0;
         const float fr = (float)std::cos(ph), fi = (float)(sg * std::sin(ph));
-        T.f16[inv][k * 32 + n] = fr;
-        T.f16[inv][k * 32 + 16 + n] = -fi;
-        T.f16[inv][(16 + k) * 32 + n] = fi;
-        T.f16[inv][(16 + k) * 32 + 16 + n] = fr;
+        f16[k][n] = fr;
+        f16[k][16 + n] = -fi;
+        f16[16 + k][n] = fi;
+        f16[16 + k][16 + n] = fr;
       }
     for (int n2 = 0; n2 < QR; ++n2)
       for (int k2 = 0; k2 < QR; ++k2) {
         const double ph = 2.0 * pi * (double)((n2 * k2) % QR) / (double)QR;
         const float fr = (float)std::cos(ph), fi = (float)(sg * std::sin(ph));
-        T.fq[inv][n2 * 32 + k2] = fr;
-        T.fq[inv][(QR + n2) * 32 + k2] = -fi;
-        T.fq[inv][n2 * 32 + QR + k2] = fi;
-        T.fq[inv][(QR + n2) * 32 + QR + k2] = fr;
+        fq[n2][k2] = fr;
+        fq[QR + n2][k2] = -fi;
+        fq[n2][QR + k2] = fi;
+        fq[QR + n2][QR + k2] = fr;
       }
+    for (int part = 0; part < 2; ++part) {
+      if (path == 0) {
+        for (int lane = 0; lane < 32; ++lane) {
+          const int g = lane >> 2, t = lane & 3;
+          for (int f = 0; f < 4; ++f) {
+            const int r = (f >> 1) * 16 + g, c = (f & 1) * 16 + 2 * t;
+            T.frag.a[inv][part][f * 32 + lane] =
+                make_uint4(pair(f16[r][c], f16[r][c + 1], part), pair(f16[r + 8][c], f16[r + 8][c + 1], part),
+                           pair(f16[r][c + 8], f16[r][c + 9], part), pair(f16[r + 8][c + 8], f16[r + 8][c + 9], part));
+          }
+          for (int kt = 0; kt < K2T; ++kt)
+            for (int nt = 0; nt < N2T; ++nt) {
+              const int n = nt * 8 + g, k = kt * 16 + 2 * t;
+              T.frag.b[inv][part][(kt * N2T + nt) * 32 + lane] =
+                  make_uint2(pair(fq[k][n], fq[k + 1][n], part), pair(fq[k + 8][n], fq[k + 9][n], part));
+            }
+        }
+      } else {
+        // 2 KiB each: b1_hi, b1_lo, b2_hi, b2_lo
+        unsigned char* img = reinterpret_cast<unsigned char*>(T.image[inv]);
+        for (int r = 0; r < 32; ++r)
+          for (int c = 0; c < 4; ++c) {
+            uint32_t v[4];
+            for (int i = 0; i < 4; ++i) v[i] = pair(f16[r][8 * c + 2 * i], f16[r][8 * c + 2 * i + 1], part);
+            std::memcpy(img + 2048 * part + umma::sw64_off(r, c), v, 16);
+            if (r >= Q2 || c >= Q2 / 8) continue;
+            for (int i = 0; i < 4; ++i) v[i] = pair(fq[8 * c + 2 * i][r], fq[8 * c + 2 * i + 1][r], part);
+            std::memcpy(img + 4096 + 2048 * part + umma::sw64_off(r, c), v, 16);
+          }
+      }
+    }
   }
 }
 
@@ -1314,6 +1358,16 @@ cudaError_t launch_dft2_tc_m(int MS, float2* buf, int count, const TcTables* tab
   }
 }
 
+// Whether the precision form's gradient kernel runs the whole V-cycle (two
+// levels or more whose bins fit a strip of 16 columns; deeper cycles take the
+// coarse kernel and the update's tail).  n = 1024, m = 256, 2500 windows, 4
+// levels: 10.6 us of coarse kernel and 8 us of the update per 64-window step
+// (sweep 5.38 -> 4.45 ms with mma.sync, 6.36 -> 5.81 with tcgen05, the tables of
+// the transforms laid out per thread included).
+bool precision_whole(const magpie_ctx* c) {
+  return c->p.levels >= 2 && !c->cnn && c->p.levels <= (c->p.m >= 128 ? Split<128>::LMAX : Split<64>::LMAX);
+}
+
 // Exit waves, tensor-core DFTs, projection, inverse DFTs and g^0 into the
 // increments (with the per-tile partial sums and the windows' corners).
 PrecArgs precision_args(magpie_ctx* c, const int32_t* idx, int count) {
@@ -1341,6 +1395,7 @@ PrecArgs precision_args(magpie_ctx* c, const int32_t* idx, int count) {
   a.wait_ns = kHandoffNs;
   a.pyr = c->pyr;
   a.L = c->p.levels;
+  a.whole = precision_whole(c);
   return a;
 }
 
@@ -1384,9 +1439,9 @@ cudaError_t launch_coarse_cycle(const PrecArgs& a, int count, int levels, cudaSt
 
 int enqueue_precision_g0(magpie_ctx* c, const PrecArgs& a, int count, cudaStream_t st) {
   switch (a.MS) {
-    case 64: CUDA_TRY(launch_precision_g0<64>(a, count, c->tabs, c->tw, st, c->precision == 2)); break;
-    case 128: CUDA_TRY(launch_precision_g0<128>(a, count, c->tabs, c->tw, st, c->precision == 2)); break;
-    case 256: CUDA_TRY(launch_precision_g0<256>(a, count, c->tabs, c->tw, st, c->precision == 2)); break;
+    case 64: CUDA_TRY(launch_precision_g0<64>(a, count, c->tabs[c->precision == 2], c->tw, st, c->precision == 2)); break;
+    case 128: CUDA_TRY(launch_precision_g0<128>(a, count, c->tabs[c->precision == 2], c->tw, st, c->precision == 2)); break;
+    case 256: CUDA_TRY(launch_precision_g0<256>(a, count, c->tabs[c->precision == 2], c->tw, st, c->precision == 2)); break;
     default: return fail(MAGPIE_EUNSUPPORTED, "the precision form needs m = 64, 128 or 256");
   }
   return MAGPIE_OK;
@@ -1417,7 +1472,7 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
     rc = enqueue_precision_g0(c, idx, count, st);
     if (!rc && c->cnn) {
       rc = enqueue_learned_tail(c, idx, count, st);
-    } else if (!rc && c->p.levels >= 2) {
+    } else if (!rc && c->p.levels >= 2 && !precision_whole(c)) {
       // the V-cycle above g^0 (g^1 and g^2 already restricted by the
       // gradient kernel): levels 1 .. L-1 on four blocks per window; the
       // finest level is formed by the update kernel as it sums the windows
@@ -1447,7 +1502,7 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
     const unsigned blocks = (unsigned)std::min<size_t>((npix + 255) / 256, 152 * 8);
     CUDA_TRY(launch_ex(accum_apply_kernel, dim3(blocks), dim3(256), 0, st, 1, true, c->z, c->acc, npix, idx, count,
                        c->p.n_pos, (const double*)c->part, step_slots(c), c->p.m, c->phi_pos, c->gn_pos));
-  } else if (c->precision && !c->cnn && c->p.levels >= 2) {
+  } else if (c->precision && !c->cnn && c->p.levels >= 2 && !precision_whole(c)) {
     // contrib holds g^0 and g1buf e^1: the update forms w . Delta from them
     ApplyArgs P = apply_args(c->z, c->p.n_rows, c->p.n_cols, c->corner, idx, count, c->p.n_pos, c->contrib,
                              c->pyr + c->M, c->p.m, c->part, c->phi_pos, c->gn_pos, c->p.m / kTcLines);
@@ -1968,7 +2023,7 @@ void magpie_destroy(magpie_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   void* bufs[] = {c->Q, c->tw, c->amp, c->stage, c->pos, c->pyr, c->pyr_q, c->pyr_u, c->contrib,
                   c->phi_pos, c->gn_pos, c->part, c->corner, c->mx, c->pnum, c->pa2, c->pmax, c->iota, c->order, c->sums, c->err,
-                  c->wz, c->lx, c->lscale, c->lacc, c->lmargin, c->lstats, c->pbuf, c->tabs, c->phase, c->g1buf,
+                  c->wz, c->lx, c->lscale, c->lacc, c->lmargin, c->lstats, c->pbuf, c->tabs[0], c->tabs[1], c->phase, c->g1buf,
                   c->g2buf, c->hand, c->acc};
   for (void* b : bufs)
     if (b) cudaFree(b);
@@ -2693,13 +2748,22 @@ int magpie_set_precision(magpie_ctx* c, int32_t mode) {
       if (e == cudaSuccess) e = cudaMalloc((void**)&c->g2buf, sizeof(float2) * (size_t)(c->M / 16) * c->p.minibatch);
       if (e == cudaSuccess) e = cudaMalloc((void**)&c->hand, sizeof(int) * 3 * (size_t)c->p.minibatch);
       if (e == cudaSuccess) e = cudaMemset(c->hand, 0, sizeof(int) * 3 * (size_t)c->p.minibatch);
-      if (e == cudaSuccess) e = cudaMalloc((void**)&c->tabs, sizeof(TcTables));
       if (e != cudaSuccess)
         return fail(e == cudaErrorMemoryAllocation ? MAGPIE_ENOMEM : MAGPIE_ECUDA,
                     std::string("precision buffers: ") + cudaGetErrorString(e));
+    }
+    TcTables*& tabs = c->tabs[mode - 1];
+    if (!tabs) {
       TcTables h;
-      build_tc_tables(m, h);
-      CUDA_TRY(cudaMemcpy(c->tabs, &h, sizeof(TcTables), cudaMemcpyHostToDevice));
+      build_tc_tables(m, mode - 1, h);
+      cudaError_t e = cudaMalloc((void**)&tabs, sizeof(TcTables));
+      if (e == cudaSuccess) e = cudaMemcpy(tabs, &h, sizeof(TcTables), cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) {
+        if (tabs) cudaFree(tabs);
+        tabs = nullptr;
+        return fail(e == cudaErrorMemoryAllocation ? MAGPIE_ENOMEM : MAGPIE_ECUDA,
+                    std::string("precision tables: ") + cudaGetErrorString(e));
+      }
     }
   }
   invalidate_graphs(c);
@@ -2717,7 +2781,7 @@ int magpie_precision_check_waits(magpie_ctx* c, double seconds) {
   a.wait_ns = (unsigned long long)(seconds * 1e9);
   const int rc = enqueue_precision_g0(c, a, count, c->stream);
   if (rc) return rc;
-  if (c->p.levels >= 3 && !c->cnn) CUDA_TRY(launch_coarse_cycle(a, count, c->p.levels, c->stream));
+  if (c->p.levels >= 3 && !c->cnn && !a.whole) CUDA_TRY(launch_coarse_cycle(a, count, c->p.levels, c->stream));
   // no update kernel runs: clear the counts here
   CUDA_TRY(cudaMemsetAsync(c->hand, 0, sizeof(int) * 3 * (size_t)count, c->stream));
   return read_err(c);
@@ -2740,7 +2804,7 @@ static int dft2_tc(const void* in, void* out, int32_t m, int32_t count, int32_t 
   if (inverse != 0 && inverse != 1) return fail(MAGPIE_EINVAL, "inverse must be 0 or 1");
   cudaStream_t st = (cudaStream_t)stream;
   TcTables h;
-  build_tc_tables(m, h);
+  build_tc_tables(m, path, h);
   std::vector<float2> htw(m);
   for (int t = 0; t < m; ++t) {
     const double ang = -2.0 * 3.14159265358979323846 * (double)t / (double)m;

@@ -20,14 +20,24 @@
 
 constexpr int kTcLines = 16;  // lines per block
 
-// Real-block DFT matrices, FP32, built on the host in float64:
+// The real-block DFT matrices (rows and columns below), built on the host in
+// float64, as the kernels consume them: already split into hi and lo FP16 and
+// laid out per thread, so that a transform loads its operands with 16-byte
+// reads instead of splitting 64 FP32 values per thread (a fifth of a
+// register-fragment transform's instructions).
 //   f16[r][c]  (32 x 32): stage 1, rows (re k1 | im k1), columns (re n1 | im n1)
 //   fq[kk][nn] (32 x 32, zero-padded): stage 2, rows (re n2 | im n2),
 //              columns (re k2 | im k2), for the Qr of the window side
 // One set for the forward (exp(-i ...)) and one for the inverse transform.
-struct TcTables {
-  float f16[2][32 * 32];
-  float fq[2][32 * 32];
+// Register fragments: a[inv][hi/lo][mt 2 + kt][lane] the stage-1 A fragments,
+// b[inv][hi/lo][kt N2T + nt][lane] the stage-2 B fragments.  tcgen05: image
+// [inv] of the operand buffers b1_hi, b1_lo, b2_hi, b2_lo (64-byte swizzle).
+union TcTables {
+  struct {
+    uint4 a[2][2][4 * 32];
+    uint2 b[2][2][8 * 32];
+  } frag;
+  uint4 image[2][512];
 };
 
 __device__ __forceinline__ uint32_t pack_f16(__half a, __half b) {
@@ -155,18 +165,11 @@ __device__ __forceinline__ void tc_lines(float* Sr, float* Si, const TcTables* _
 
   // ---- stage-1 operands: the 16-point DFT matrix as A fragments (hi, lo)
   uint32_t ah[2][2][4], al[2][2][4];
-  {
-    const float* F = tabs->f16[INV];
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int kt = 0; kt < 2; ++kt) {
-        const int r = mt * 16 + g, c = kt * 16 + 2 * t;
-        split2(F[r * 32 + c], F[r * 32 + c + 1], ah[mt][kt][0], al[mt][kt][0]);
-        split2(F[(r + 8) * 32 + c], F[(r + 8) * 32 + c + 1], ah[mt][kt][1], al[mt][kt][1]);
-        split2(F[r * 32 + c + 8], F[r * 32 + c + 9], ah[mt][kt][2], al[mt][kt][2]);
-        split2(F[(r + 8) * 32 + c + 8], F[(r + 8) * 32 + c + 9], ah[mt][kt][3], al[mt][kt][3]);
-      }
+  for (int f = 0; f < 4; ++f) {
+    const uint4 h = __ldg(&tabs->frag.a[INV][0][f * 32 + lane]), w = __ldg(&tabs->frag.a[INV][1][f * 32 + lane]);
+    ah[f >> 1][f & 1][0] = h.x, ah[f >> 1][f & 1][1] = h.y, ah[f >> 1][f & 1][2] = h.z, ah[f >> 1][f & 1][3] = h.w;
+    al[f >> 1][f & 1][0] = w.x, al[f >> 1][f & 1][1] = w.y, al[f >> 1][f & 1][2] = w.z, al[f >> 1][f & 1][3] = w.w;
   }
   __syncthreads();
 
@@ -219,17 +222,15 @@ __device__ __forceinline__ void tc_lines(float* Sr, float* Si, const TcTables* _
 
   // ---- stage 2: rows (line, k1), NL * 16 of them; the Qr-point DFT matrix as B fragments
   uint32_t bh2[K2T][N2T][2], bl2[K2T][N2T][2];
-  {
-    const float* F = tabs->fq[INV];
 #pragma unroll
-    for (int kt = 0; kt < K2T; ++kt)
+  for (int kt = 0; kt < K2T; ++kt)
 #pragma unroll
-      for (int nt = 0; nt < N2T; ++nt) {
-        const int n = nt * 8 + g, k = kt * 16 + 2 * t;
-        split2(F[k * 32 + n], F[(k + 1) * 32 + n], bh2[kt][nt][0], bl2[kt][nt][0]);
-        split2(F[(k + 8) * 32 + n], F[(k + 9) * 32 + n], bh2[kt][nt][1], bl2[kt][nt][1]);
-      }
-  }
+    for (int nt = 0; nt < N2T; ++nt) {
+      const uint2 h = __ldg(&tabs->frag.b[INV][0][(kt * N2T + nt) * 32 + lane]);
+      const uint2 w = __ldg(&tabs->frag.b[INV][1][(kt * N2T + nt) * 32 + lane]);
+      bh2[kt][nt][0] = h.x, bh2[kt][nt][1] = h.y;
+      bl2[kt][nt][0] = w.x, bl2[kt][nt][1] = w.y;
+    }
   constexpr int MT2 = NL * 16 / 16, PER2 = MT2 / 4;  // m-tiles of 16 rows = one line each
   float out[PER2][N2T][4];
 #pragma unroll
@@ -355,24 +356,13 @@ __device__ __forceinline__ void tc_lines_umma(float* Sr, float* Si, const TcTabl
   const int tid = threadIdx.x;
   const uint32_t trow = U.tmem + ((uint32_t)(tid & ~31) << 16);  // this warp's TMEM lanes
   const float sx = tc_scale(mx), out_scale = scale / sx;  // its barrier: the lines in place
-  // B operands: stage 1 rows r, K c: f16[r][c]; stage 2 rows nn, K kk: fq[kk][nn] (0 in the padding)
-  {
-    const float* F1 = tabs->f16[INV];
-    const int r = tid >> 2, c = tid & 3;
-    float v[8];
+  // B operands: stage 1 rows r, K c: f16[r][c]; stage 2 rows nn, K kk: fq[kk][nn]
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = F1[r * 32 + 8 * c + k];
-    put_chunk(U.b1_hi, U.b1_lo, r, c, v);
-    const float* F2 = tabs->fq[INV];
-    if (tid < Q2 * (Q2 / 8)) {
-      const int r2 = tid / (Q2 / 8), c2 = tid % (Q2 / 8);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int kk = 8 * c2 + k;
-        v[k] = kk < 2 * QR && r2 < 2 * QR ? F2[kk * 32 + r2] : 0.f;
-      }
-      put_chunk(U.b2_hi, U.b2_lo, r2, c2, v);
-    }
+  for (int i = 0; i < 4; ++i) {
+    const uint4 v = __ldg(&tabs->image[INV][tid + 128 * i]);
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(U.b1_hi + 16u * (uint32_t)(tid + 128 * i)), "r"(v.x),
+                 "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
   }
   __syncthreads();  // the lines in place
 
@@ -550,6 +540,7 @@ struct PrecArgs {
   unsigned long long wait_ns;  // bound of each hand-off wait
   const float* pyr;    // level factors (window-kernel layout)
   int L;               // levels
+  int whole;           // the gradient kernel runs the whole V-cycle (its bins fit the block's strip)
 };
 
 // The three window-phase kernels of a minibatch step.  Each block takes
@@ -561,7 +552,9 @@ struct PrecArgs {
 //                               sum of (|Psi| - sqrt d)^2), inverse DFT
 //   grad_dft_kernel    columns: inverse DFT, g^0 = conj(Q)(R - Q z_k) into the
 //                               increments (+ the tile's sum of |g^0|^2), and
-//                               for two levels or more g^1 = W_u^0 . I(g^0)
+//                               for two levels or more g^1 = W_u^0 . I(g^0);
+//                               with at most Split::LMAX levels the whole
+//                               V-cycle, whose increments it writes instead
 // The window buffer holds psi's column transforms, then R's row transforms.
 
 // Window hand-off between the step's kernels.  Each transform kernel lets
@@ -771,14 +764,25 @@ __global__ void __launch_bounds__(128, TcSm<MS>::template min_blocks<PATH>()) gr
         g = make_float2(qq.x * dx + qq.y * dy, qq.x * dy - qq.y * dx);
       }
       gn += g.x * g.x + g.y * g.y;
-      out[(size_t)p * MS + c] = g;
+      if (!A.whole) out[(size_t)p * MS + c] = g;
       Sr[S::at(l, p)] = g.x;
       Si[S::at(l, p)] = g.y;
     }
   }
   const double s = block_sum((double)gn, red, threadIdx.x, 128);  // also the barrier before g^1
   if (threadIdx.x == 0) A.part[((size_t)B.w * A.T + B.tile) * 2 + 1] = B.ok ? s : 0.0;
-  if (A.g1) {
+  if (A.whole) {
+    // every level's bins lie in the block's 16 columns: the increments
+    // themselves, strip by strip in registers (split_vcycle), instead of
+    // g^1 and g^2 for a coarse kernel and an update that reads e^1 as well
+    constexpr int E = Split<MS>::E;
+    static_assert(NL == Split<MS>::NL, "strips of the split form");
+    const int l = threadIdx.x % NL, c = B.l0 + l;
+    const auto Y = [&](int r, int j) { return make_float2(Sr[S::at(j, r)], Si[S::at(j, r)]); };
+    const auto put = [&](int r, int cc, float2 v) { out[(size_t)r * MS + cc] = v; };
+#pragma unroll 1
+    for (int s0 = threadIdx.x / NL; s0 < MS / E; s0 += 128 / NL) split_vcycle_levels<MS>(A.L, Y, A.pyr, l, c, s0 * E, put);
+  } else if (A.g1) {
     // the block's NL / 2 bin columns, every bin row; the four g^0 of a bin
     // summed row by row
     constexpr int NB = (NL / 2) * h / 128;  // bins per thread

@@ -173,14 +173,15 @@ __device__ __forceinline__ void split_project_body(const StepArgs& A, int win, i
 // half-warp owns column c, the thread the strip's E rows from R0 on.  Level-j
 // values are held by all 2^j lanes of their bin, so a restriction is one or
 // two shuffles and the whole cycle stays in registers.
-template <int MS, int L, class Sink>
-__device__ __forceinline__ void split_vcycle(const float2* Y, const float* pyr, int l, int c, int R0, const Sink& put) {
-  constexpr int E = Split<MS>::E, NL = Split<MS>::NL;
+// Y(r, l): g^0 at row r of the block's column l.
+template <int MS, int L, class Src, class Sink>
+__device__ __forceinline__ void split_vcycle(const Src& Y, const float* pyr, int l, int c, int R0, const Sink& put) {
+  constexpr int E = Split<MS>::E;
   float2 g[E];  // level j's E >> j values at offset E - (E >> (j - 1))
   constexpr auto off = [](int j) { return E - (E >> (j - 1)); };
 #pragma unroll
   for (int a = 0; a < E / 2; ++a) {
-    float2 v = cadd(Y[(R0 + 2 * a) * NL + l], Y[(R0 + 2 * a + 1) * NL + l]);
+    float2 v = cadd(Y(R0 + 2 * a, l), Y(R0 + 2 * a + 1, l));
     v = cadd(v, shfl_xor2(v, 1));
     g[a] = cscale_rn(v, 0.25f * __ldg(&pyr[lvl_off(MS, 1) + (R0 / 2 + a) * (MS / 2) + (c >> 1)]));
   }
@@ -216,9 +217,22 @@ __device__ __forceinline__ void split_vcycle(const float2* Y, const float* pyr, 
 #pragma unroll
   for (int a = 0; a < E; ++a) {
     const float u = __ldg(&pyr[(R0 + a) * MS + c]);
-    const float2 g0 = Y[(R0 + a) * NL + l], e = g[a >> 1];
+    const float2 g0 = Y(R0 + a, l), e = g[a >> 1];
     put(R0 + a, c, f2(__fmaf_rn(u, e.x, g0.x), __fmaf_rn(u, e.y, g0.y)));
   }
+}
+
+template <int MS, class Src, class Sink>
+__device__ __forceinline__ void split_vcycle_levels(int levels, const Src& Y, const float* pyr, int l, int c, int R0,
+                                                    const Sink& put) {
+  if (levels == 2)
+    split_vcycle<MS, 2>(Y, pyr, l, c, R0, put);
+  else if (levels == 3)
+    split_vcycle<MS, 3>(Y, pyr, l, c, R0, put);
+  else if (Split<MS>::LMAX == 4 || levels == 4)
+    split_vcycle<MS, 4>(Y, pyr, l, c, R0, put);
+  else
+    split_vcycle<MS, Split<MS>::LMAX>(Y, pyr, l, c, R0, put);
 }
 
 template <int MS, bool ATOM>
@@ -280,15 +294,8 @@ __device__ __forceinline__ void split_grad_body(const StepArgs& A, int win, int 
   }
   split_sum<S::T>(gn2, A.part + (size_t)(win * S::TILES + tile) * 2 + 1);  // its barrier: g^0 in place
   if (direct) return;
-  const int R0 = g * E;
-  if (A.levels == 2)
-    split_vcycle<MS, 2>(X, A.pyr, l, c, R0, put);
-  else if (A.levels == 3)
-    split_vcycle<MS, 3>(X, A.pyr, l, c, R0, put);
-  else if (S::LMAX == 4 || A.levels == 4)
-    split_vcycle<MS, 4>(X, A.pyr, l, c, R0, put);
-  else
-    split_vcycle<MS, S::LMAX>(X, A.pyr, l, c, R0, put);
+  split_vcycle_levels<MS>(
+      A.levels, [&](int r, int j) { return X[r * NL + j]; }, A.pyr, l, c, g * E, put);
 }
 
 // One problem.  Each kernel waits for the one before, then lets the next
