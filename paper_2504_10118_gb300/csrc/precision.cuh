@@ -40,16 +40,13 @@ union TcTables {
   uint4 image[2][512];
 };
 
-__device__ __forceinline__ uint32_t pack_f16(__half a, __half b) {
-  __half2 v = __halves2half2(a, b);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
-
-// hi and lo FP16 pairs of (a, b)
+// hi and lo FP16 pairs of (a, b), by the paired conversions
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-  const __half ha = __float2half_rn(a), hb = __float2half_rn(b);
-  hi = pack_f16(ha, hb);
-  lo = pack_f16(__float2half_rn(a - __half2float(ha)), __float2half_rn(b - __half2float(hb)));
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
 __device__ __forceinline__ void mma_f16(float* c, const uint32_t* a, const uint32_t* b) {
@@ -201,7 +198,22 @@ __device__ __forceinline__ void tc_lines(float* Sr, float* Si, const TcTables* _
       for (int kt = 0; kt < 2; ++kt) mma3(acc[i][mt], ah[mt][kt], al[mt][kt], bh[kt], bl[kt]);
   }
   __syncthreads();
-  // twiddle w_m^{+-n2 k1}; thread holds re/im of k1 = g, g+8 for columns 2t, 2t+1
+  // twiddle w_m^{+-n2 k1}; thread holds re/im of k1 = g, g+8 for columns 2t, 2t+1.
+  // Its columns' n2 repeat every NV tiles (PER1 tiles of a warp start at a
+  // multiple of Qr), so at most eight twiddles serve them all.
+  constexpr int NV = QR > 8 ? QR / 8 : 1;
+  static_assert((PER1 * 8) % QR == 0, "a warp's columns are whole lines");
+  float2 wt[NV][2][2];
+#pragma unroll
+  for (int v = 0; v < NV; ++v)
+#pragma unroll
+    for (int cc = 0; cc < 2; ++cc)
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        float2 w = __ldg(&tw[(((v * 8 + 2 * t + cc) % QR) * (g + 8 * hh)) % MS]);
+        if (INV) w.y = -w.y;
+        wt[v][cc][hh] = w;
+      }
 #pragma unroll
   for (int i = 0; i < PER1; ++i)
 #pragma unroll
@@ -212,8 +224,7 @@ __device__ __forceinline__ void tc_lines(float* Sr, float* Si, const TcTables* _
       for (int hh = 0; hh < 2; ++hh) {
         const int k1 = g + 8 * hh;
         const float yr = acc[i][0][2 * hh + cc], yi = acc[i][1][2 * hh + cc];
-        float2 w = tw[(n2 * k1) % MS];
-        if (INV) w.y = -w.y;
+        const float2 w = wt[i % NV][cc][hh];
         Sr[S::at(l, k1 * QR + n2)] = yr * w.x - yi * w.y;
         Si[S::at(l, k1 * QR + n2)] = yr * w.y + yi * w.x;
       }
@@ -246,15 +257,16 @@ __device__ __forceinline__ void tc_lines(float* Sr, float* Si, const TcTables* _
       uint32_t a_h[4], a_l[4];
       float v[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int row = g + ((q >> 1) & 1) * 8;
-        const int kk = kt * 16 + 2 * t + (q & 1) + ((q >> 2) & 1) * 8;
-        float val = 0.f;
+      for (int q = 0; q < 4; ++q) {  // pairs of consecutive columns: one 8-byte read each
+        const int row = g + (q & 1) * 8;
+        const int kk = kt * 16 + 2 * t + (q >> 1) * 8;
+        float2 val = make_float2(0.f, 0.f);
         if (kk < QR)
-          val = Sr[S::at(l, row * QR + kk)];
+          val = *reinterpret_cast<const float2*>(&Sr[S::at(l, row * QR + kk)]);
         else if (kk < 2 * QR)
-          val = Si[S::at(l, row * QR + kk - QR)];
-        v[q] = val;
+          val = *reinterpret_cast<const float2*>(&Si[S::at(l, row * QR + kk - QR)]);
+        v[2 * q] = val.x;
+        v[2 * q + 1] = val.y;
       }
 #pragma unroll
       for (int r = 0; r < 4; ++r) split2(v[2 * r], v[2 * r + 1], a_h[r], a_l[r]);
@@ -496,8 +508,8 @@ template <int MS, int AXIS, int INV, int PATH>
 __global__ void __launch_bounds__(128) dft_tc_kernel(float2* __restrict__ data, const TcTables* __restrict__ tabs,
                                                      const float2* __restrict__ tw, float scale, int* err) {
   using S = TcSm<MS>;
-  __shared__ float Sr[S::NL * S::LD];
-  __shared__ float Si[S::NL * S::LD];
+  __shared__ __align__(8) float Sr[S::NL * S::LD];
+  __shared__ __align__(8) float Si[S::NL * S::LD];
   TcPath<PATH> T;
   T.begin();
   const int tiles = MS / S::NL;
@@ -625,8 +637,8 @@ template <int MS, int PATH>
 __global__ void __launch_bounds__(128, TcSm<MS>::template min_blocks<PATH>()) exit_dft_kernel(const PrecArgs A, const TcTables* __restrict__ tabs,
                                                        const float2* __restrict__ tw) {
   using S = TcSm<MS>;
-  __shared__ float Sr[S::NL * S::LD];
-  __shared__ float Si[S::NL * S::LD];
+  __shared__ __align__(8) float Sr[S::NL * S::LD];
+  __shared__ __align__(8) float Si[S::NL * S::LD];
   grid_dep_wait();  // launched as a programmatic dependent of the step's last kernel before
   grid_dep_launch();
   TcPath<PATH> T;
@@ -658,8 +670,8 @@ template <int MS, int PATH>
 __global__ void __launch_bounds__(128, TcSm<MS>::template min_blocks<PATH>()) project_dft_kernel(const PrecArgs A, const TcTables* __restrict__ tabs,
                                                           const float2* __restrict__ tw) {
   using S = TcSm<MS>;
-  __shared__ float Sr[S::NL * S::LD];
-  __shared__ float Si[S::NL * S::LD];
+  __shared__ __align__(8) float Sr[S::NL * S::LD];
+  __shared__ __align__(8) float Si[S::NL * S::LD];
   __shared__ double red[4];
   grid_dep_launch();  // the exit kernel's windows are handed off one by one
   TcPath<PATH> T;
@@ -698,12 +710,19 @@ __global__ void __launch_bounds__(128, TcSm<MS>::template min_blocks<PATH>()) pr
       const float vx = Sr[S::at(l, p)], vy = Si[S::at(l, p)];
       const float a = av[u];
       const float n2 = vx * vx + vy * vy;
-      const float mag = sqrtf(n2);
+      // |Psi| and 1 / |Psi| from one reciprocal square root with a Newton step
+      // (within an ulp, where a square root and two divisions took half of the
+      // projection's instructions); left out where n2 overflowed
+      float rs = rsqrtf(n2);
+      const float er = fmaf(-0.5f * n2 * rs, rs, 0.5f);
+      const bool fin = n2 <= 3.402823466e38f;
+      if (fin) rs = fmaf(rs, er, rs);
+      const float mag = fin ? (n2 > 0.f ? n2 * rs : 0.f) : n2;
       const float d = mag - a;
       res += d * d;
       float2 ph = make_float2(1.f, 0.f);  // theta(0) = 0
       if (n2 > 0.f) {
-        ph = make_float2(vx / mag, vy / mag);
+        ph = make_float2(vx * rs, vy * rs);
         if (A.phase && B.ok) A.phase[(size_t)B.k * MS * MS + o] = ph;
       } else if (A.phase && B.ok) {
         ph = A.phase[(size_t)B.k * MS * MS + o];  // Eq. (specification): the previous visit's phase
@@ -727,8 +746,8 @@ __global__ void __launch_bounds__(128, TcSm<MS>::template min_blocks<PATH>()) gr
                                                        const float2* __restrict__ tw) {
   using S = TcSm<MS>;
   constexpr int NL = S::NL, h = MS / 2;
-  __shared__ float Sr[NL * S::LD];
-  __shared__ float Si[NL * S::LD];
+  __shared__ __align__(8) float Sr[NL * S::LD];
+  __shared__ __align__(8) float Si[NL * S::LD];
   __shared__ double red[4];
   grid_dep_launch();  // the project kernel's windows are handed off one by one
   TcPath<PATH> T;
