@@ -90,17 +90,19 @@ __global__ void __launch_bounds__(256) apply_tail_kernel(ApplyArgs P) {
 // Several problems in one launch (1-D grid): problem i owns blocks
 // table[i].block0 .. table[i + 1].block0 - 1.
 template <int TW, int TH>
-__global__ void __launch_bounds__(256) apply_kernel_batched(const ApplyArgs* __restrict__ table, int n) {
+__global__ void __launch_bounds__(256) apply_kernel_batched(const ApplyArgs* __restrict__ table, int n,
+                                                            int first) {
+  const int blk = (int)blockIdx.x + first;  // the launch may start inside a step's table
   int lo = 0, hi = n - 1;
-  while (lo < hi) {  // last problem whose first block is <= blockIdx.x
+  while (lo < hi) {  // last problem whose first block is <= blk
     const int mid = (lo + hi + 1) >> 1;
-    if (table[mid].block0 <= (int)blockIdx.x)
+    if (table[mid].block0 <= blk)
       lo = mid;
     else
       hi = mid - 1;
   }
   const ApplyArgs& P = table[lo];
-  const int t = (int)blockIdx.x - P.block0;
+  const int t = blk - P.block0;
   apply_body<TW, TH>(P, t % P.tiles_x, t / P.tiles_x);
 }
 
@@ -351,13 +353,14 @@ __global__ void __launch_bounds__(1024) reduce_kernel(const double* part, int CL
                                                       double* gn_pos, double* out) {
   __shared__ double red[32];
   double a = 0.0, b = 0.0;
+  const double scale = 0.5 / ((double)MS * (double)MS);  // a power of two
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     double pk = 0.0, gk = 0.0;
     for (int q = 0; q < CL; ++q) {
       pk += part[(size_t)(k * CL + q) * 2];
       gk += part[(size_t)(k * CL + q) * 2 + 1];
     }
-    pk /= 2.0 * (double)MS * (double)MS;
+    pk *= scale;
     gk = sqrt(gk);
     phi_pos[k] = pk;
     gn_pos[k] = gk;
@@ -616,6 +619,8 @@ struct GroupApplyLaunch {
   int n;          // problems in the launch
   int blocks;     // total tiles
   int max_count;  // largest window count (shared memory)
+  int first = 0;  // blocks of the step's table before this launch's
+  int ms = 0;     // window side of its problems (0: any)
 };
 // One launch of the persistent form: the members of one window side at one
 // batched step, their windows and then their update tiles.
@@ -677,7 +682,8 @@ struct magpie_group {
   int2* map = nullptr;          // cluster -> (table entry, window slot)
   ApplyArgs* atable[3] = {};    // per apply tile shape: one entry per (batched step, member)
   std::vector<std::vector<GroupWindowLaunch>> wl;  // per batched step
-  std::vector<GroupApplyLaunch> al[3];             // per apply tile shape, per batched step
+  std::vector<GroupApplyLaunch> al[3];             // per apply tile shape, per batched step (its problems by side)
+  std::vector<std::vector<GroupApplyLaunch>> als[3];  // the same, one launch per window side
   std::vector<ApplyArgs> atable_host[3];           // host copies (the autotuner's scratch tables)
   cudaGraphExec_t graph = nullptr;
   // autotuner: register bound (blocks per SM) of the batched window kernel
@@ -825,8 +831,10 @@ StepArgs make_args(magpie_ctx* c, const int32_t* idx) {
 
 // Whether the context's minibatch steps take the split form of the window
 // phase: every plain or learned step with windows of 64 and more whose levels
-// fit a strip.  The probe step and the phase rule keep the cluster kernel.  us
-// per step, three levels, ordered update (split / cluster kernel):
+// fit a strip.  The probe step and the phase rule keep the cluster kernel, and
+// so do m = 64 minibatches beyond 64 windows that still run at once on two
+// blocks per SM (152 clusters of two).  us per step, three levels, ordered
+// update (split / cluster kernel):
 //   m = 64, n = 300   B = 16: 9.8 / 10.8, 64: 11.9 / 12.2, 128: 15.4 / 14.4, 512: 35.7 / 47.3
 //   m = 128, n = 512  B = 4: 11.3 / 14.9, 16: 14.9 / 16.7, 64: 20.7 / 22.0, 256: 57.8 / 66.7
 //   m = 256, n = 800  B = 4: 16.6 / 27.3, 16: 27.1 / 50.0, 64: 57.9 / 117
@@ -835,6 +843,7 @@ StepArgs make_args(magpie_ctx* c, const int32_t* idx) {
 // both forms, the FP64 sums of Phi_k and ||g|| are taken in another order).
 bool split_form(const magpie_ctx* c) {
   const int m = c->p.m;
+  if (m == 64 && c->p.minibatch > 64 && c->p.minibatch <= 152) return false;
   return m >= 64 && c->p.levels <= (m >= 128 ? Split<128>::LMAX : Split<64>::LMAX) && !c->p.update_probe &&
          !c->precision && !(c->variant & 2) && !c->stamps;
 }
@@ -1603,12 +1612,19 @@ int capture_sweep(magpie_ctx* c, cudaGraphExec_t* out) {
   return MAGPIE_OK;
 }
 
-// Replays (capturing it on first use) the graph of one sweep over the
-// permutation already in c->order.
+// One sweep over the permutation already in c->order: replays its graph.  The
+// first sweep of a context is launched step by step, and its graph is captured
+// while the GPU runs it (first sweep of the n = 512, m = 128, 900-window
+// problem, which waited for capture and instantiation before: 441 -> 332 us).
 int launch_sweep(magpie_ctx* c) {
   if (!c->graph) {
-    const int rc = capture_sweep(c, &c->graph);
-    if (rc) return rc;
+    const int N = c->p.n_pos, B = c->p.minibatch;
+    for (int s = 0; s < N; s += B) {
+      // the first step's predecessor is the copy of the permutation itself
+      const int rc = enqueue_step(c, c->order + s, std::min(B, N - s), c->stream, nullptr, s > 0);
+      if (rc) return rc;
+    }
+    return capture_sweep(c, &c->graph);
   }
   CUDA_TRY(cudaGraphLaunch(c->graph, c->stream));
   return MAGPIE_OK;
@@ -1729,9 +1745,8 @@ cudaError_t launch_group_windows(magpie_group* g, const GroupWindowLaunch& L, cu
   return launch_window_batched_m<kStep>(L.ms, g->table, g->map + L.map_off, L.windows, st, minb);
 }
 
-// The window phases of batched step t: the window sides run concurrently,
-// forked from `st` onto the group's side streams and joined back (a group of
-// 12 uneven problems: 2.74 ms per sweep, the sides one after another 2.96).
+// The window phases of batched step t, the window sides concurrent: forked
+// from `st` onto the group's side streams and joined back.
 int enqueue_group_windows(magpie_group* g, size_t t, cudaStream_t st) {
   const auto& Ls = g->wl[t];
   bool several = false;
@@ -1753,17 +1768,41 @@ int enqueue_group_windows(magpie_group* g, size_t t, cudaStream_t st) {
 
 // The update of batched step t with apply tile shape v, from the device table
 // `table` (default: the group's own table of that shape).
-cudaError_t launch_apply_batched(magpie_group* g, int v, int t, cudaStream_t st, const ApplyArgs* table = nullptr) {
-  const GroupApplyLaunch& A = g->al[v][t];
+cudaError_t launch_apply_batched(magpie_group* g, int v, const GroupApplyLaunch& A, cudaStream_t st,
+                                 const ApplyArgs* table = nullptr) {
   const ApplyArgs* tab = table ? table : g->atable[v] + A.tab_off;
   const size_t smem = sizeof(ApplyEntry) * A.max_count;
-  switch (v) {
-    case 0: apply_kernel_batched<16, 16><<<A.blocks, 256, smem, st>>>(tab, A.n); break;
-    case 1: apply_kernel_batched<32, 8><<<A.blocks, 256, smem, st>>>(tab, A.n); break;
-    case 2: apply_kernel_batched<32, 32><<<A.blocks, 256, smem, st>>>(tab, A.n); break;
-    default: return cudaErrorInvalidValue;
+  void (*const k[3])(const ApplyArgs*, int, int) = {apply_kernel_batched<16, 16>, apply_kernel_batched<32, 8>,
+                                                    apply_kernel_batched<32, 32>};
+  return launch_ex(k[v], dim3((unsigned)A.blocks), dim3(256), smem, st, 1, true, tab, A.n, A.first);
+}
+
+// One sweep as separate launches: the members of a window side advance from
+// step to step (windows, then update) on a stream of their own, since nothing
+// but the sweep's ends ties the sides together; a side with few windows left
+// then runs beside the others instead of between them (12 uneven problems:
+// 2.60 ms per sweep, 2.73 with the sides joined after every step, 2.51 with the
+// update also listing its windows before the gradient kernel ends).
+int enqueue_group_sweep(magpie_group* g, cudaStream_t st) {
+  std::vector<int> sides;  // every member has a first step, so step 0 has them all
+  for (const auto& L : g->wl[0])
+    if (sides.empty() || sides.back() != L.ms) sides.push_back(L.ms);
+  if (sides.size() > 1) CUDA_TRY(cudaEventRecord(g->fork, st));
+  for (size_t j = 0; j < sides.size(); ++j) {
+    cudaStream_t s = j == 0 ? st : g->side[j];
+    if (j) CUDA_TRY(cudaStreamWaitEvent(s, g->fork, 0));
+    for (size_t t = 0; t < g->wl.size(); ++t) {
+      for (const auto& L : g->wl[t])
+        if (L.ms == sides[j]) CUDA_TRY(launch_group_windows(g, L, s, g->minb[ilog2(L.ms) - 3]));
+      for (const auto& A : g->als[g->apply_shape][t])
+        if (A.ms == sides[j]) CUDA_TRY(launch_apply_batched(g, g->apply_shape, A, s));
+    }
   }
-  return cudaGetLastError();
+  for (size_t j = 1; j < sides.size(); ++j) {
+    CUDA_TRY(cudaEventRecord(g->join[j], g->side[j]));
+    CUDA_TRY(cudaStreamWaitEvent(st, g->join[j], 0));
+  }
+  return MAGPIE_OK;
 }
 
 // Times every apply tile shape on batched step 0 (one warm-up, then three
@@ -1788,9 +1827,9 @@ int group_tune_apply(magpie_group* g, cudaStream_t st, cudaEvent_t e0, cudaEvent
       off += (size_t)P.n_rows * P.n_cols;
     }
     e = cudaMemcpyAsync(tab, at.data(), sizeof(ApplyArgs) * at.size(), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_apply_batched(g, v, 0, st, tab);
+    if (e == cudaSuccess) e = launch_apply_batched(g, v, g->al[v][0], st, tab);
     if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-    for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = launch_apply_batched(g, v, 0, st, tab);
+    for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = launch_apply_batched(g, v, g->al[v][0], st, tab);
     if (e == cudaSuccess) e = cudaEventRecord(e1, st);
     if (e == cudaSuccess) e = cudaEventSynchronize(e1);
     float ms = 0.f;
@@ -1892,7 +1931,7 @@ int group_tune_form(magpie_group* g, cudaStream_t st, cudaEvent_t e0, cudaEvent_
     if (form == 0) {
       const int wrc = enqueue_group_windows(g, 0, st);
       if (wrc) return wrc;
-      CUDA_TRY(launch_apply_batched(g, g->apply_shape, 0, st, atab));
+      CUDA_TRY(launch_apply_batched(g, g->apply_shape, A, st, atab));
       return MAGPIE_OK;
     }
     CUDA_TRY(cudaMemsetAsync(g->qbuf, 0, sizeof(int) * g->qbuf_n, st));
@@ -2413,20 +2452,30 @@ int magpie_group_create(magpie_group** out, magpie_ctx* const* ctxs, int32_t n, 
     for (int v = 0; v < 3; ++v) {
       std::vector<ApplyArgs>& at = g->atable_host[v];
       GroupApplyLaunch A{(int)at.size(), 0, 0, 0};
-      for (int i = 0; i < n; ++i) {
+      std::vector<GroupApplyLaunch> sides;
+      for (int k = 0; k < 6 * n; ++k) {  // member k % n, the members side by side
+        const int i = k % n;
         magpie_ctx* c = g->members[i];
-        if (entry[i] < 0) continue;
+        if (entry[i] < 0 || c->p.m != 8 << (k / n)) continue;
+        if (sides.empty() || sides.back().ms != c->p.m)
+          sides.push_back(GroupApplyLaunch{(int)at.size(), 0, 0, 0, A.blocks, c->p.m});
         const int cnt = std::min(c->p.minibatch, c->p.n_pos - t * c->p.minibatch);
         ApplyArgs P = apply_args(c->z, c->p.n_rows, c->p.n_cols, c->corner, c->order + (size_t)t * c->p.minibatch,
                                  cnt, c->p.n_pos, c->contrib, c->pyr + c->M, c->p.m, c->part, c->phi_pos,
                                  c->gn_pos, step_slots(c), kApplyShapes[v]);
+        P.early = split_form(c) ? 1 : 0;
         P.block0 = A.blocks;
         A.blocks += apply_tiles(P);
         A.max_count = std::max(A.max_count, cnt);
         ++A.n;
+        GroupApplyLaunch& S = sides.back();
+        S.blocks = A.blocks - S.first;
+        S.max_count = std::max(S.max_count, cnt);
+        ++S.n;
         at.push_back(P);
       }
       g->al[v].push_back(A);
+      g->als[v].push_back(sides);
     }
   }
   auto upload = [&](void** dst, const void* src, size_t bytes) -> int {
@@ -2494,10 +2543,7 @@ int magpie_group_sweep(magpie_group* g, const int32_t* const* orders) {
       for (size_t t = 0; t < g->pl.size() && e == cudaSuccess && !rc; ++t)
         rc = enqueue_persistent_step(g, t, g->cap_stream, g->ptable, 0);
     } else {
-      for (size_t t = 0; t < g->wl.size() && e == cudaSuccess && !rc; ++t) {
-        rc = enqueue_group_windows(g, t, g->cap_stream);
-        if (!rc) e = launch_apply_batched(g, g->apply_shape, t, g->cap_stream);
-      }
+      rc = enqueue_group_sweep(g, g->cap_stream);
     }
     cudaError_t e2 = cudaStreamEndCapture(g->cap_stream, &gr);
     if (rc) {

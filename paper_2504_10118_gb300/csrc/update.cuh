@@ -52,6 +52,7 @@ struct ApplyEntry {
 
 // Phi_k and ||grad Phi_k|| of the step's windows from the block partials, in block order.
 __device__ __forceinline__ void apply_partials(const ApplyArgs& P) {
+  const double scale = 0.5 / ((double)P.MS * (double)P.MS);  // a power of two
   for (int b = threadIdx.x; b < P.count; b += blockDim.x) {
     const int k = P.idx[b];
     if ((unsigned)k >= (unsigned)P.n_pos) continue;
@@ -60,7 +61,7 @@ __device__ __forceinline__ void apply_partials(const ApplyArgs& P) {
       a += P.part[(size_t)(b * P.slots + q) * 2];
       g += P.part[(size_t)(b * P.slots + q) * 2 + 1];
     }
-    P.phi_pos[k] = a / (2.0 * (double)P.MS * (double)P.MS);
+    P.phi_pos[k] = a * scale;
     P.gn_pos[k] = sqrt(g);
   }
 }
@@ -87,10 +88,13 @@ __device__ __forceinline__ void apply_body(const ApplyArgs& P, const int tx, con
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int r0 = R0 + (int)(threadIdx.x / TW), c = C0 + (int)(threadIdx.x % TW);
   float2 zz[PPT];
+  const auto load_z = [&]() {
 #pragma unroll
-  for (int p = 0; p < PPT; ++p)
-    zz[p] = (r0 + p * RS < P.n_rows && c < P.n_cols) ? __ldcg(&P.z[(size_t)(r0 + p * RS) * P.n_cols + c])
-                                                      : make_float2(0.f, 0.f);
+    for (int p = 0; p < PPT; ++p)
+      zz[p] = (r0 + p * RS < P.n_rows && c < P.n_cols) ? __ldcg(&P.z[(size_t)(r0 + p * RS) * P.n_cols + c])
+                                                        : make_float2(0.f, 0.f);
+  };
+  if (P.early) load_z();
   // windows meeting this tile, listed in minibatch order: every warp takes
   // 32 consecutive windows per round, ballots, and the rounds are stitched
   // together by per-warp counts
@@ -119,6 +123,8 @@ __device__ __forceinline__ void apply_body(const ApplyArgs& P, const int tx, con
     grid_dep_wait();
     grid_dep_launch();
   }
+  if (nl == 0) return;
+  if (!P.early) load_z();  // beside the first increments, and not in a tile without windows
   float nx[PPT], ny[PPT], d[PPT];
 #pragma unroll
   for (int p = 0; p < PPT; ++p) nx[p] = ny[p] = d[p] = 0.f;
