@@ -68,6 +68,9 @@ cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
 // the window kernel in mode `mode` (a Mode) over `windows` windows;
 template <int MS>
 cudaError_t window_launch(int mode, const StepArgs& a, int windows, cudaStream_t st);
+// a sweep's step of small windows (MS <= 32) that lets its update start early;
+template <int MS>
+cudaError_t window_early_launch(const StepArgs& a, int windows, cudaStream_t st);
 // forward intensities of windows 0 .. windows - 1 (tw: MS twiddles, host);
 template <int MS>
 cudaError_t window_sim_launch(const StepArgs& a, const float2* tw, int windows, cudaStream_t st);

@@ -528,6 +528,15 @@ cudaError_t launch_window_batched_m(int MS, const StepArgs* table, const int2* m
   }
 }
 
+cudaError_t launch_window_early_m(int MS, const StepArgs& a, int windows, cudaStream_t st) {
+  switch (MS) {
+    case 8: return window_early_launch<8>(a, windows, st);
+    case 16: return window_early_launch<16>(a, windows, st);
+    case 32: return window_early_launch<32>(a, windows, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 cudaError_t launch_sim_m(int MS, const StepArgs& a, const float2* tw, int windows, cudaStream_t st) {
   switch (MS) {
 #define MAGPIE_CASE(S) \
@@ -1473,7 +1482,13 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
   // 21.0; m = 256, B = 64: 70.9 against 63.7; m = 64, B = 16: 10.3 against
   // 9.8, B = 64: 11.8 against 11.9, B = 256: 20.5 against 21.7)
   const bool split = split_form(c);
-  const bool atom = c->acc && !c->precision && !c->cnn && !a.phase &&
+  // a sweep's small windows, up to 64 of 32 x 32: the update lists them while
+  // they run (us per step, early / not: m = 32, n = 400: B = 8 6.7 / 7.4, 32 7.7 /
+  // 8.7, 64 8.9 / 9.2, 128 9.8 / 9.2; m = 16: B = 16 6.2 / 6.7, 256 7.7 / 8.2),
+  // which also serves deterministic = 0 better than the atomics (B = 32: 9.2)
+  const bool early = own_idx && c->p.m <= 32 && (long long)c->p.minibatch * c->M <= 65536 && !a.phase && !c->cnn &&
+                     !c->p.update_probe && !c->precision && !c->stamps;
+  const bool atom = c->acc && !early && !c->precision && !c->cnn && !a.phase &&
                     (!split || (c->p.m == 64 && c->p.minibatch >= 64));
   if (ev) CUDA_TRY(cudaEventRecord(ev[0], st));
   int rc = MAGPIE_OK;
@@ -1498,6 +1513,8 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
     } else if (atom) {
       a.acc = c->acc;
       CUDA_TRY(launch_window_m<kStepAtomic>(c->p.m, a, count, st));
+    } else if (early) {
+      CUDA_TRY(launch_window_early_m(c->p.m, a, count, st));
     } else {
       CUDA_TRY(launch_window_m<kStep>(c->p.m, a, count, st));
     }
@@ -1528,7 +1545,8 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
       P.hand = c->hand;
       P.nhand = 3 * count;
     }
-    P.early = split ? 1 : 0;
+    P.early = split ? 1 : early ? 2 : 0;
+    P.pos = c->pos;
     CUDA_TRY(launch_apply_args(P, st));
   }
   if (c->p.update_probe) {

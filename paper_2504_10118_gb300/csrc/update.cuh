@@ -40,8 +40,10 @@ struct ApplyArgs {
   const float* u0;         // [MS][MS] u^0
   int* hand;               // precision form: the step's window hand-off counts, zeroed by
   int nhand;               // block (0, 0) once the grid may run (null otherwise)
-  int early;               // the object and the corners are final before the stream's previous kernel
-                           // ends (split form): the windows are listed before the wait for it
+  int early;               // the object and the windows' positions are final before the stream's previous
+                           // kernel ends: the windows are listed before the wait for it, their corners
+                           // as an earlier kernel recorded them (1) or from idx and pos (2)
+  const int32_t* pos;      // [n_pos][2] (early = 2)
 };
 
 // One window of a tile's list: its corner, the offset of its increments less
@@ -104,7 +106,13 @@ __device__ __forceinline__ void apply_body(const ApplyArgs& P, const int tx, con
     bool hit = false;
     int2 q = make_int2(0, 0);
     if (b < count) {
-      q = __ldcg(&P.corners[b]);
+      if (P.early == 2) {
+        const int k = P.idx[b];
+        q = (unsigned)k < (unsigned)P.n_pos ? make_int2(P.pos[2 * k], P.pos[2 * k + 1])
+                                            : make_int2(-(1 << 30), -(1 << 30));
+      } else {
+        q = __ldcg(&P.corners[b]);
+      }
       hit = q.x < R0 + TH && q.x + MS > R0 && q.y < C0 + TW && q.y + MS > C0;
     }
     const unsigned mask = __ballot_sync(0xffffffffu, hit);

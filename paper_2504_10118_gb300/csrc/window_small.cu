@@ -7,4 +7,7 @@ namespace magpie_impl {
 MAGPIE_INSTANTIATE_WINDOW(8)
 MAGPIE_INSTANTIATE_WINDOW(16)
 MAGPIE_INSTANTIATE_WINDOW(32)
+MAGPIE_INSTANTIATE_EARLY(8)
+MAGPIE_INSTANTIATE_EARLY(16)
+MAGPIE_INSTANTIATE_EARLY(32)
 }  // namespace magpie_impl
