@@ -351,15 +351,23 @@ __global__ void __launch_bounds__(256) probe_apply_kernel(float2* Q, int M, cons
 // order (one block).
 __global__ void __launch_bounds__(1024) reduce_kernel(const double* part, int CL, int MS, int n, double* phi_pos,
                                                       double* gn_pos, double* out) {
-  __shared__ double red[32];
+  __shared__ double red[2][32];
   double a = 0.0, b = 0.0;
   const double scale = 0.5 / ((double)MS * (double)MS);  // a power of two
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    double pk = 0.0, gk = 0.0;
-    for (int q = 0; q < CL; ++q) {
-      pk += part[(size_t)(k * CL + q) * 2];
-      gk += part[(size_t)(k * CL + q) * 2 + 1];
+    double pv[kMaxCluster], gv[kMaxCluster];  // every block's partials in flight together
+#pragma unroll
+    for (int q = 0; q < kMaxCluster; ++q) {
+      pv[q] = q < CL ? part[(size_t)(k * CL + q) * 2] : 0.0;
+      gv[q] = q < CL ? part[(size_t)(k * CL + q) * 2 + 1] : 0.0;
     }
+    double pk = 0.0, gk = 0.0;
+#pragma unroll
+    for (int q = 0; q < kMaxCluster; ++q)
+      if (q < CL) {
+        pk += pv[q];
+        gk += gv[q];
+      }
     pk *= scale;
     gk = sqrt(gk);
     phi_pos[k] = pk;
@@ -367,18 +375,20 @@ __global__ void __launch_bounds__(1024) reduce_kernel(const double* part, int CL
     a += pk;
     b += gk;
   }
-  const int T = blockDim.x, tid = threadIdx.x;
-  for (int pass = 0; pass < 2; ++pass) {
-    double v = pass ? b : a;
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_down_sync(0xffffffffu, a, o);
+    b += __shfl_down_sync(0xffffffffu, b, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = a;
+    red[1][threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x < 64) {  // one warp per sum
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    double v = l < (int)(blockDim.x / 32) ? red[w][l] : 0.0;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    if (tid == 0) {
-      double r = 0.0;
-      for (int i = 0; i < T / 32; ++i) r += red[i];
-      out[pass] = r;
-    }
-    __syncthreads();
+    if (l == 0) out[w] = v;
   }
 }
 
