@@ -40,6 +40,9 @@ TRAFFIC_FILES = {1: os.path.join(ROOT, "profiles", "window_kernel_m128_mid.txt")
                  0: os.path.join(ROOT, "profiles", "window_kernel_atomic_m128_mid.txt")}
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2504_10118_gb300", "csrc", f)
                   for f in ("fft_lines.cuh", "window_kernel.cuh", "window_body.inc")]
+# the same of the split form's three kernels (windows of 64 and more)
+SPLIT_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "split_kernels_m128_mid.txt")
+SPLIT_SOURCES = [os.path.join(ROOT, "paper_2504_10118_gb300", "csrc", f) for f in ("fft_lines.cuh", "window_split.cuh")]
 
 
 def flops_per_window(m: int) -> float:
@@ -124,21 +127,21 @@ def peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0}, "fallback"
 
 
-def kernel_source_hash() -> str:
+def kernel_source_hash(sources=None) -> str:
     """sha256 over the window kernel's source files (the ncu figures go stale
-    when it changes)."""
+    when it changes), or over the given ones."""
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES:
+    for f in sources or KERNEL_SOURCES:
         h.update(open(f, "rb").read())
     return h.hexdigest()
 
 
-def measured_traffic(deterministic: int = 1):
-    """DRAM bytes per launch of the window kernel (of the given update) from
-    the committed ncu summary, or None when the kernel source changed since it
-    was taken."""
+def measured_traffic(deterministic: int = 1, split: bool = False):
+    """DRAM bytes per launch of the window kernel (of the given update), or of
+    the split form's three kernels, from the committed ncu summary, or None
+    when the kernel source changed since it was taken."""
     try:
-        lines = open(TRAFFIC_FILES[deterministic]).read().splitlines()
+        lines = open(SPLIT_TRAFFIC_FILE if split else TRAFFIC_FILES[deterministic]).read().splitlines()
     except OSError:
         return None
     kv = {}
@@ -146,7 +149,7 @@ def measured_traffic(deterministic: int = 1):
         if ":" in ln:
             k, v = ln.split(":", 1)
             kv[k.strip()] = v.strip()
-    src = kernel_source_hash()
+    src = kernel_source_hash(SPLIT_SOURCES if split else None)
     if kv.get("source_sha256") != src or "dram_bytes_per_launch" not in kv:
         return None
     return float(kv["dram_bytes_per_launch"])
@@ -400,7 +403,8 @@ def batched_measure(dev, magpie, warmup: int, steps: int, pg=None, clocks=None):
     magpie.magpie_group_set_persistent(group, persistent)
     steps_max = max(math.ceil(w.n_pos / w.minibatch) for w in ws)
     sides = [len({w.m for w in ws if math.ceil(w.n_pos / w.minibatch) > t}) for t in range(steps_max)]
-    launches = sum(sides) if persistent else sum(n + 1 for n in sides)
+    # separate launches: per step and side three window-phase kernels and an update
+    launches = sum(sides) if persistent else sum(4 * n for n in sides)
     tuning = magpie.magpie_group_tuning(group)
     shape, shapes = magpie.magpie_group_apply_tuning(group)
     group.close()
@@ -720,6 +724,25 @@ def launches_per_step(args, w) -> int:
     return 2
 
 
+def split_form(w) -> bool:
+    """Whether the FP32 form's steps of this workload run as the three strip kernels."""
+    return w.m >= 64 and w.levels <= (5 if w.m >= 128 else 4) and not (w.m == 64 and 64 < w.minibatch <= 152)
+
+
+def step_launches(args, w) -> int:
+    """launches_per_step with the library's forms for this workload: windows of
+    64 and more run their window phase as three kernels, the precision form's
+    gradient kernel runs V-cycles of up to five levels (four at m = 64) itself,
+    and the network's first two layers need neither a cast nor a split-K sum."""
+    n = launches_per_step(args, w)
+    fits = w.m >= 64 and w.levels <= (5 if w.m >= 128 else 4)
+    if args.learned:
+        return n + (2 if split_form(w) else 0) - 2
+    if args.dft in ("tc", "tcgen05"):
+        return n - (1 if w.levels >= 3 and fits else 0)
+    return n + (2 if split_form(w) else 0)
+
+
 def tensor_roofline(args, w, windows, wk_ms, ap_ms, prof_sweeps, launches, pk, src):
     """Roofline of the tensor-core work of the precision or learned form over
     its window phase (every kernel between the window's exit wave and the
@@ -814,7 +837,7 @@ def run_ours(args, w):
     alu_peak, alu_src = fp32_peak(dev, magpie)
     achieved_tf = windows * flops_per_window(w.m) / (wk_ms * 1e-3) / 1e12
     achieved_gbs = windows * hbm_bytes_per_window(w.m) / (wk_ms * 1e-3) / 1e9
-    traffic = measured_traffic(det) if fp32_form else None
+    traffic = measured_traffic(det, split_form(w)) if fp32_form else None
 
     # the other update of the FP32 form on the same data, timed the same way
     update_ab = None
@@ -838,7 +861,8 @@ def run_ours(args, w):
                                                      "window_kernel_ms_per_sweep": wk2 / prof_sweeps,
                                                      "update_kernel_ms_per_sweep": ap2 / prof_sweeps}}
         update_ab = dict(rec, headline=args.update,
-                         note="same data and sweep orders; per-kernel times from event-bracketed launches")
+                         note="same data and sweep orders; per-kernel times from event-bracketed launches; windows "
+                              "of 128 and more take the ordered update for both values of the parameter")
 
     # end to end through the host-buffer call: order + intensities in, object out
     order_h = [torch.from_numpy(synth.make_order(w.n_pos, 1000 + s)).pin_memory() for s in range(max(2, args.steps))]
@@ -898,7 +922,8 @@ def run_ours(args, w):
             "learned": learned_rec,
             "roofline": ({"bound": "alu", "achieved": achieved_tf, "peak": alu_peak, "unit": "TFLOP/s",
                          "frac": achieved_tf / alu_peak, "traffic": traffic,
-                         "kernel": f"window_kernel<{w.m}, {'step' if det else 'step_atomic'}>",
+                         "kernel": (f"split_exit/project/grad_kernel<{w.m}> (one window phase)" if split_form(w)
+                                    else f"window_kernel<{w.m}, {'step' if det else 'step_atomic'}>"),
                          "avg_launch_ms": wk_ms / max(launches, 1),
                          "flops_per_window": flops_per_window(w.m),
                          "peak_source": alu_src,
@@ -916,7 +941,7 @@ def run_ours(args, w):
                     "call": "magpie_sweep_host_async x steps, then magpie_sync: every sweep copies its order "
                             "and the whole intensity set in (pinned host buffers, on a copy stream while the "
                             "previous sweep computes) and the object out"},
-            "gpu_launches": launches_per_step(args, w) * math.ceil(w.n_pos / w.minibatch) * args.steps,
+            "gpu_launches": step_launches(args, w) * math.ceil(w.n_pos / w.minibatch) * args.steps,
             "clocks": clk,
         }
         print(json.dumps(line), flush=True)

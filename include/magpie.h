@@ -93,8 +93,9 @@ typedef struct {
  *      accumulators (16 n_rows n_cols bytes) with 16-byte float atomics, and a
  *      streaming kernel applies N / D and clears them: faster, but the
  *      order of the floating-point sums varies from run to run.
- * The atomic update serves the FP32 window kernel (with or without the probe
- * step); the precision form, the learned correction, the phase rule of
+ * With deterministic = 0 the library may take the ordered update where that is
+ * the faster of the two (windows of 128 and more, and small minibatches).  The
+ * atomic update serves the FP32 window kernel (with or without the probe step); the precision form, the learned correction, the phase rule of
  * Eq. (specification) and context groups always use the ordered update.
  */
 
@@ -151,7 +152,8 @@ int magpie_step(magpie_ctx* ctx, const int32_t* idx, int32_t count);
  * over consecutive slices of order[0..n_pos-1] (DEVICE int32 permutation),
  * the last slice possibly shorter.  The order is copied to the context
  * first, so the caller may reuse its buffer once the stream reaches the
- * call.  The steps replay a CUDA graph captured on the first call.
+ * call.  The steps replay a CUDA graph captured behind the first call's own
+ * launches.
  */
 int magpie_sweep(magpie_ctx* ctx, const int32_t* order);
 
@@ -248,10 +250,11 @@ int magpie_forward_intensities(const void* object, int32_t n_rows, int32_t n_col
  * Context groups: several independent reconstructions advanced together.
  * magpie_group_sweep is one sweep of every member, exactly as magpie_sweep
  * on each of them (member results are bitwise those of separate sweeps), but
- * batched: batched step t runs step t of every member that has one, all
- * windows of equal m in one launch and all members' object updates in one
- * more (or, in the persistent form below, one launch per m for windows and
- * updates together), replayed from one CUDA graph.  Members may differ in
+ * batched: the members of one window side m advance together, step t's
+ * windows of all that have one in one launch (three for sides of 64 and more)
+ * and their object updates in one more, the sides concurrently (or, in the
+ * persistent form below, one launch per m and step for windows and updates
+ * together), replayed from one CUDA graph.  Members may differ in
  * every size.
  *   ctxs   : n contexts created on the current device, none with
  *            update_probe = 1, each at most once; they must outlive the group
@@ -314,7 +317,9 @@ int magpie_group_set_apply_shape(magpie_group* group, int32_t shape);
  *      magpie_group_status reports MAGPIE_ETIMEOUT.
  * Both forms sum each pixel's windows in minibatch order and give bitwise
  * identical objects.  magpie_group_create times batched step 0 in both forms
- * (updates writing scratch copies of the objects) and uses the faster.
+ * (updates writing scratch copies of the objects) and uses the faster; a group
+ * with a member whose own sweeps run as three launches per step stays with
+ * separate launches, whose per-window values equal that member's bit for bit.
  * magpie_group_form_tuning reports the form in use (*persistent) and the two
  * measured ms per batched step 0 (ms[2], HOST); magpie_group_set_persistent
  * forces one (MAGPIE_EINVAL unless 0 or 1).  magpie_group_set_wait_limit sets

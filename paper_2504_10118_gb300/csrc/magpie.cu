@@ -1,16 +1,18 @@
 // magpie.cu -- MAGPIE sweep on one GB300 (sm_103a): kernels and the C ABI.
 //
-// Per minibatch step, one thread block per scan window k runs, entirely in
-// shared memory and registers:
+// Per minibatch step, every scan window k goes through
 //   pass A  gather z_k, exit wave Q . z_k, column FFTs          (Section 2.1)
 //   pass B  row FFTs, Fourier modulus projection onto sqrt(d_k),
 //           inverse row FFTs                                    (Definition REW)
 //   pass C  inverse column FFTs -> R_k, then g = conj(Q)(R_k - Q z_k)
 //   pass D  the MAGPS V-cycle (Algorithm MAGPS) in residual form
-// and writes its increment w . Delta_k (w = u + |Q|^2) to a per-window
-// buffer.  A second kernel then updates every object pixel by the ordered
-// sum over the minibatch, z += sum_k w.Delta_k / sum_k w, so no atomics are
-// used and results are bitwise reproducible.
+// and leaves its increment w . Delta_k (w = u + |Q|^2) in a per-window buffer:
+// in one kernel, a cluster of blocks per window (window_kernel.cuh), or in
+// three kernels over strips of 16 lines with the window in L2 between them
+// (window_split.cuh), the same bits either way.  Another kernel then updates
+// every object pixel by the ordered sum over the minibatch,
+// z += sum_k w.Delta_k / sum_k w, so no atomics are used and results are
+// bitwise reproducible.
 //
 // Residual form of Algorithm MAGPS.  With the weights of Eq. (def_weights),
 // W_R . Q = (I_H^h Q_H) . W_z, so by Lemma (commutative) the coarse residual
@@ -489,19 +491,25 @@ ApplyArgs apply_args(float2* z, int n_rows, int n_cols, const int2* corners, con
 // blocks of one update: its tiles and the block of the partial sums
 int apply_tiles(const ApplyArgs& P) { return P.tiles_x * P.tiles_y + 1; }
 
-// The update of one problem on its own, in 32 x 32 tiles (four pixels per
-// thread share the window list and its tests) once those are 400 or more, else
-// in 16 x 16 tiles, which keep small objects from leaving SMs idle: step of 64
-// windows with m = 128 (us, 16 x 16 / 32 x 32 tiles): 19.8 / 21.7 at n = 512,
-// 22.6 / 22.1 at 640, 26.1 / 22.6 at 1024; m = 256: 62.6 / 68.0 at n = 600,
-// 63.5 / 62.5 at 768.  The precision form's tail does as well with either.
+// The update of one problem on its own, in the largest of 32 x 32, 32 x 16 and
+// 16 x 16 tiles (four, two and one pixel per thread, which share the window
+// list and its tests) that leaves at least five blocks per SM: smaller grids
+// leave SMs idle.  us per 64-window step, three levels, in that order:
+//   m = 128: n = 512 24.4 / 20.3 / 19.6, 640 23.3 / 21.0 / 21.6, 1024 22.1 / 23.6 / 25.6
+//   m = 256: n = 600 70.9 / 58.3 / 57.7, 1024 56.9 / 56.9 / 59.5 (four levels)
 cudaError_t launch_apply_args(ApplyArgs P, cudaStream_t st) {
-  const long long big = (long long)((P.n_cols + 31) / 32) * ((P.n_rows + 31) / 32);
-  const ApplyShape s = kApplyShapes[big >= 400 ? 2 : 0];
-  P.tiles_x = (P.n_cols + s.tw - 1) / s.tw;
-  P.tiles_y = (P.n_rows + s.th - 1) / s.th;
-  return launch_ex(big >= 400 ? apply_kernel<32, 32> : apply_kernel<16, 16>, dim3((unsigned)apply_tiles(P)), dim3(256),
-                   sizeof(ApplyEntry) * P.count, st, 1, true, P);
+  struct Tile {
+    int w, h;
+    void (*k)(ApplyArgs);
+  };
+  const Tile tiles[3] = {{32, 32, apply_kernel<32, 32>}, {32, 16, apply_kernel<32, 16>}, {16, 16, apply_kernel<16, 16>}};
+  const Tile* t = tiles;
+  for (;; ++t) {
+    P.tiles_x = (P.n_cols + t->w - 1) / t->w;
+    P.tiles_y = (P.n_rows + t->h - 1) / t->h;
+    if (t == tiles + 2 || (long long)P.tiles_x * P.tiles_y >= 5 * 152) break;
+  }
+  return launch_ex(t->k, dim3((unsigned)apply_tiles(P)), dim3(256), sizeof(ApplyEntry) * P.count, st, 1, true, P);
 }
 
 cudaError_t launch_apply(float2* z, int n_rows, int n_cols, const int2* corners, const int32_t* idx, int count,
@@ -592,7 +600,7 @@ void minb_candidates(int MS, int* c) {
 
 cudaError_t prepare_kernels(int MS) {
   cudaError_t e = cudaSuccess;
-  for (auto* k : {apply_kernel<16, 16>, apply_kernel<32, 32>, apply_tail_kernel})
+  for (auto* k : {apply_kernel<16, 16>, apply_kernel<32, 16>, apply_kernel<32, 32>, apply_tail_kernel})
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(sizeof(ApplyEntry) * kMaxMinibatch));
@@ -1388,10 +1396,10 @@ cudaError_t launch_dft2_tc_m(int MS, float2* buf, int count, const TcTables* tab
 
 // Whether the precision form's gradient kernel runs the whole V-cycle (two
 // levels or more whose bins fit a strip of 16 columns; deeper cycles take the
-// coarse kernel and the update's tail).  n = 1024, m = 256, 2500 windows, 4
-// levels: 10.6 us of coarse kernel and 8 us of the update per 64-window step
-// (sweep 5.38 -> 4.45 ms with mma.sync, 6.36 -> 5.81 with tcgen05, the tables of
-// the transforms laid out per thread included).
+// coarse kernel and the update's tail; same bits either way).  n = 1024,
+// m = 256, 2500 windows, 4 levels: the coarse kernel's 10.6 us and 8 us of the
+// update per 64-window step (sweep, with the pre-split tables: 5.37 -> 4.51 ms
+// with mma.sync, 6.35 -> 5.89 with tcgen05).
 bool precision_whole(const magpie_ctx* c) {
   return c->p.levels >= 2 && !c->cnn && c->p.levels <= (c->p.m >= 128 ? Split<128>::LMAX : Split<64>::LMAX);
 }

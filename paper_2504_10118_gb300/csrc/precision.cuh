@@ -710,19 +710,12 @@ __global__ void __launch_bounds__(128, TcSm<MS>::template min_blocks<PATH>()) pr
       const float vx = Sr[S::at(l, p)], vy = Si[S::at(l, p)];
       const float a = av[u];
       const float n2 = vx * vx + vy * vy;
-      // |Psi| and 1 / |Psi| from one reciprocal square root with a Newton step
-      // (within an ulp, where a square root and two divisions took half of the
-      // projection's instructions); left out where n2 overflowed
-      float rs = rsqrtf(n2);
-      const float er = fmaf(-0.5f * n2 * rs, rs, 0.5f);
-      const bool fin = n2 <= 3.402823466e38f;
-      if (fin) rs = fmaf(rs, er, rs);
-      const float mag = fin ? (n2 > 0.f ? n2 * rs : 0.f) : n2;
+      const float mag = sqrtf(n2);
       const float d = mag - a;
       res += d * d;
       float2 ph = make_float2(1.f, 0.f);  // theta(0) = 0
       if (n2 > 0.f) {
-        ph = make_float2(vx * rs, vy * rs);
+        ph = make_float2(vx / mag, vy / mag);
         if (A.phase && B.ok) A.phase[(size_t)B.k * MS * MS + o] = ph;
       } else if (A.phase && B.ok) {
         ph = A.phase[(size_t)B.k * MS * MS + o];  // Eq. (specification): the previous visit's phase
@@ -800,7 +793,7 @@ __global__ void __launch_bounds__(128, TcSm<MS>::template min_blocks<PATH>()) gr
     const auto Y = [&](int r, int j) { return make_float2(Sr[S::at(j, r)], Si[S::at(j, r)]); };
     const auto put = [&](int r, int cc, float2 v) { out[(size_t)r * MS + cc] = v; };
 #pragma unroll 1
-    for (int s0 = threadIdx.x / NL; s0 < MS / E; s0 += 128 / NL) split_vcycle_levels<MS>(A.L, Y, A.pyr, l, c, s0 * E, put);
+    for (int s0 = threadIdx.x / NL; s0 < MS / E; s0 += 128 / NL) split_vcycle_levels<MS, true>(A.L, Y, A.pyr, l, c, s0 * E, put);
   } else if (A.g1) {
     // the block's NL / 2 bin columns, every bin row; the four g^0 of a bin
     // summed row by row

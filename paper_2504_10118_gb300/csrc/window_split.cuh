@@ -173,16 +173,30 @@ __device__ __forceinline__ void split_project_body(const StepArgs& A, int win, i
 // half-warp owns column c, the thread the strip's E rows from R0 on.  Level-j
 // values are held by all 2^j lanes of their bin, so a restriction is one or
 // two shuffles and the whole cycle stays in registers.
-// Y(r, l): g^0 at row r of the block's column l.
-template <int MS, int L, class Src, class Sink>
+// Y(r, l): g^0 at row r of the block's column l.  PREC: the precision form's
+// roundings (its coarse kernel's: every bin summed row by row, and the other
+// product of the up-pass fused), so that its results do not depend on whether
+// the levels fit a strip.
+template <int MS, int L, bool PREC, class Src, class Sink>
 __device__ __forceinline__ void split_vcycle(const Src& Y, const float* pyr, int l, int c, int R0, const Sink& put) {
   constexpr int E = Split<MS>::E;
   float2 g[E];  // level j's E >> j values at offset E - (E >> (j - 1))
   constexpr auto off = [](int j) { return E - (E >> (j - 1)); };
+  // ((x00 + x01) + x10) + x11 of a bin, this lane holding one column (p, q) of it
+  const auto rows = [&](float2 p, float2 q, int x) {
+    const float2 r0 = cadd(p, shfl_xor2(p, x)), o = shfl_xor2(q, x);
+    const bool left = (l & x) == 0;
+    return cadd(cadd(r0, left ? q : o), left ? o : q);
+  };
 #pragma unroll
   for (int a = 0; a < E / 2; ++a) {
-    float2 v = cadd(Y(R0 + 2 * a, l), Y(R0 + 2 * a + 1, l));
-    v = cadd(v, shfl_xor2(v, 1));
+    float2 v;
+    if (PREC) {
+      v = rows(Y(R0 + 2 * a, l), Y(R0 + 2 * a + 1, l), 1);
+    } else {
+      v = cadd(Y(R0 + 2 * a, l), Y(R0 + 2 * a + 1, l));
+      v = cadd(v, shfl_xor2(v, 1));
+    }
     g[a] = cscale_rn(v, 0.25f * __ldg(&pyr[lvl_off(MS, 1) + (R0 / 2 + a) * (MS / 2) + (c >> 1)]));
   }
 #pragma unroll
@@ -191,7 +205,9 @@ __device__ __forceinline__ void split_vcycle(const Src& Y, const float* pyr, int
     for (int a = 0; a < (E >> j); ++a) {
       const float2 p = g[off(j - 1) + 2 * a], q = g[off(j - 1) + 2 * a + 1];
       float2 v;
-      if (j == 2) {
+      if (PREC) {
+        v = rows(p, q, 1 << (j - 1));
+      } else if (j == 2) {
         v = cadd(p, q);
         v = cadd(v, shfl_xor2(v, 2));
       } else {  // the window kernel sums these bins row by row
@@ -210,6 +226,8 @@ __device__ __forceinline__ void split_vcycle(const Src& Y, const float* pyr, int
     for (int a = 0; a < (E >> j); ++a) {
       if (j == L - 1)
         g[off(j) + a] = cscale_rn(g[off(j) + a], __ldg(iw + a * n));
+      else if (PREC)  // prolong with u^l / w^l e^{l+1} as the fused product
+        g[off(j) + a] = prolong(g[off(j + 1) + (a >> 1)], __ldg(rr + a * n), __ldg(iw + a * n), g[off(j) + a]);
       else
         g[off(j) + a] = prolong(g[off(j) + a], __ldg(iw + a * n), __ldg(rr + a * n), g[off(j + 1) + (a >> 1)]);
     }
@@ -222,17 +240,17 @@ __device__ __forceinline__ void split_vcycle(const Src& Y, const float* pyr, int
   }
 }
 
-template <int MS, class Src, class Sink>
+template <int MS, bool PREC, class Src, class Sink>
 __device__ __forceinline__ void split_vcycle_levels(int levels, const Src& Y, const float* pyr, int l, int c, int R0,
                                                     const Sink& put) {
   if (levels == 2)
-    split_vcycle<MS, 2>(Y, pyr, l, c, R0, put);
+    split_vcycle<MS, 2, PREC>(Y, pyr, l, c, R0, put);
   else if (levels == 3)
-    split_vcycle<MS, 3>(Y, pyr, l, c, R0, put);
+    split_vcycle<MS, 3, PREC>(Y, pyr, l, c, R0, put);
   else if (Split<MS>::LMAX == 4 || levels == 4)
-    split_vcycle<MS, 4>(Y, pyr, l, c, R0, put);
+    split_vcycle<MS, 4, PREC>(Y, pyr, l, c, R0, put);
   else
-    split_vcycle<MS, Split<MS>::LMAX>(Y, pyr, l, c, R0, put);
+    split_vcycle<MS, Split<MS>::LMAX, PREC>(Y, pyr, l, c, R0, put);
 }
 
 template <int MS, bool ATOM>
@@ -294,7 +312,7 @@ __device__ __forceinline__ void split_grad_body(const StepArgs& A, int win, int 
   }
   split_sum<S::T>(gn2, A.part + (size_t)(win * S::TILES + tile) * 2 + 1);  // its barrier: g^0 in place
   if (direct) return;
-  split_vcycle_levels<MS>(
+  split_vcycle_levels<MS, false>(
       A.levels, [&](int r, int j) { return X[r * NL + j]; }, A.pyr, l, c, g * E, put);
 }
 

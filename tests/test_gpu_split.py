@@ -81,11 +81,12 @@ def test_skipped_index_and_raw_intensities():
         c.close()
 
 
-def test_large_update_tiles_and_atomics():
-    """An object with 400 or more 32 x 32 tiles is updated in those, a group
-    forced to 16 x 16 tiles gives the same bits; the float atomics that m = 64
-    keeps for minibatches of 64 and more agree to rounding."""
-    mb = Member((645, 64, 12, 50, 5, 3, 64), 5)
+@pytest.mark.parametrize("n,step", [(645, 50), (897, 70)])
+def test_large_update_tiles_and_atomics(n, step):
+    """Objects large enough for 760 tiles of 32 x 16 or of 32 x 32 are updated in
+    those, a group forced to 16 x 16 tiles gives the same bits; the float
+    atomics that m = 64 keeps for minibatches of 64 and more agree to rounding."""
+    mb = Member((n, 64, 12, step, 5, 3, 64), 5)
     alone = mb.ctx()
     z_alone = mb.zt
     member = mb.ctx()
