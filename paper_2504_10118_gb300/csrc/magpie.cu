@@ -948,8 +948,9 @@ ConvPlan conv_plan_tc(const ConvFwd& a) {
 }
 
 // Split of a batch's backward pass: per layer 1 .. 4 the weight gradient's
-// tiles and pixel chunks (enough blocks for two per SM, at least 128 pixels
-// per chunk), the blocks of layers 0 and 5, and where each keeps its partial
+// tiles and pixel chunks (enough blocks for three per SM, which the kernels'
+// shared memory allows, at least 128 pixels per chunk; 236 us per 64-window
+// gradient, 239 and 240 with two and one), the blocks of layers 0 and 5, and where each keeps its partial
 // sums.
 struct GradPlan {
   int wm[kCnnLayers], wn[kCnnLayers], chunk[kCnnLayers], chunks[kCnnLayers];
@@ -972,7 +973,7 @@ GradPlan grad_plan(int h, int B) {
       g.wm[l] = M / 64;
       g.wn[l] = (N + 63) / 64;
       const int tiles = g.wm[l] * g.wn[l];
-      const int want = std::max(1, std::min((2 * 152 + tiles - 1) / tiles, K / 128));
+      const int want = std::max(1, std::min((3 * 152 + tiles - 1) / tiles, K / 128));
       g.chunk[l] = ((K + want - 1) / want + 31) / 32 * 32;
       g.chunks[l] = (K + g.chunk[l] - 1) / g.chunk[l];
       g.stride[l] = (size_t)M * N + M;
@@ -1123,7 +1124,8 @@ int cnn_enqueue_backward(magpie_cnn* n, const float* dy, float* grad, cudaStream
     a.oplane = pixels(l) * L.cin;
     a.out_f32 = l == 1;
     a.rows = up ? (int)pixels(l) : B * ho * ho;
-    const int bm = l == 3 ? 32 : 64, bn = l == 1 ? 32 : 64;  // layer 3's longest class is 64 steps: narrower tiles
+    // layer 3's longest class is 64 steps: narrower tiles (239 against 251 us)
+    const int bm = l == 3 ? 32 : 64, bn = l == 1 ? 32 : 64;
     a.xm = (a.rows + bm - 1) / bm;
     a.xn = L.cin / bn;
     a.xblocks = a.xm * a.xn * (up ? 1 : 4);
