@@ -123,7 +123,10 @@ __device__ __forceinline__ void split_project_body(const StepArgs& A, int win, i
   __shared__ float2 X[NL * MS];
   const int tid = threadIdx.x, rl = tid / G, g = tid % G, kr = tile * NL + rl;
   const int k = A.idx[win];
-  if ((unsigned)k >= (unsigned)A.n_pos) return;
+  if ((unsigned)k >= (unsigned)A.n_pos) {
+    grid_dep_wait();  // see split_exit_kernel
+    return;
+  }
   const float* ampr = A.amp + (size_t)k * S::M + kr * MS + g;
   float av[E];  // fetched while the exit kernel finishes
 #pragma unroll
@@ -260,7 +263,10 @@ __device__ __forceinline__ void split_grad_body(const StepArgs& A, int win, int 
   __shared__ float2 X[NL * MS];
   const int tid = threadIdx.x, l = tid % NL, g = tid / NL, c = tile * NL + l;
   const int k = A.idx[win];
-  if ((unsigned)k >= (unsigned)A.n_pos) return;
+  if ((unsigned)k >= (unsigned)A.n_pos) {
+    grid_dep_wait();  // see split_exit_kernel
+    return;
+  }
   const int pr = A.pos[2 * k], pc = A.pos[2 * k + 1];
   const float2* zp = A.z + (size_t)(pr + g) * A.n_cols + pc + c;
   const float2* qp = A.Q + g * MS + c;
@@ -316,9 +322,13 @@ __device__ __forceinline__ void split_grad_body(const StepArgs& A, int win, int 
       A.levels, [&](int r, int j) { return X[r * NL + j]; }, A.pyr, l, c, g * E, put);
 }
 
-// One problem.  Each kernel waits for the one before, then lets the next
-// one's blocks be set up, so that a kernel's blocks start once every kernel
-// but the one before theirs has ended.
+// One problem.  Every block of a kernel waits for the kernel before, also
+// where its window is skipped, then lets the next one's blocks be set up, so
+// that a kernel's blocks start once every kernel but the one before theirs has
+// ended: the update reads the corners that the exit kernel wrote before its
+// own wait, which is for the gradient kernel.  (A grid that ended without
+// having waited, as one of skipped windows alone once did, would let the
+// update read the corners of an earlier step.)
 template <int MS>
 __global__ void __launch_bounds__(Split<MS>::T, Split<MS>::MB[0]) split_exit_kernel(const __grid_constant__ StepArgs A, bool early) {
   split_exit_body<MS>(A, blockIdx.x / Split<MS>::TILES, blockIdx.x % Split<MS>::TILES, early);
