@@ -78,7 +78,10 @@ __global__ void __launch_bounds__(256) apply_kernel(ApplyArgs P) {
     grid_dep_wait();
     clear_handoff(P);
   }
-  apply_body<TW, TH>(P, blockIdx.x % P.tiles_x, blockIdx.x / P.tiles_x);
+  // a single problem's 16 x 16 tiles all fit on the GPU beside the gradient
+  // kernel's blocks: those without windows wait like the others (290.4 us per
+  // sweep at n = 512, m = 128; 292.8 if they leave at once)
+  apply_body<TW, TH, 256, false, (TW * TH > 256)>(P, blockIdx.x % P.tiles_x, blockIdx.x / P.tiles_x);
 }
 
 // The precision form's update: the same ordered sum, each window's
