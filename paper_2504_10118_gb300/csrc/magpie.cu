@@ -69,19 +69,24 @@ __device__ __forceinline__ void clear_handoff(const ApplyArgs& P) {
 }
 
 // One problem: a block per tile and one for the partial sums.
-// Launched as a programmatic dependent of the window kernel (its blocks, let
-// in early, would slow the next window kernel: 0.328 against 0.319 ms per
-// sweep, so it does not trigger its dependents).
+// Launched as a programmatic dependent of the window phase.  Behind the split
+// form and a sweep's small windows (early) it lets the next step's first kernel
+// be set up once its own wait is over; behind the cluster kernel it does not,
+// whose blocks, let in early, slow it (0.328 against 0.319 ms per sweep).
 template <int TW, int TH>
 __global__ void __launch_bounds__(256) apply_kernel(ApplyArgs P) {
   if (P.hand) {
     grid_dep_wait();
     clear_handoff(P);
   }
+  // The partial sums, the longest chain of loads, go first: behind 1024 tiles
+  // their block ended a step of 8 windows of 16 x 16 at n = 512 half a
+  // microsecond late (6.4 us, 5.9 this way).
+  const int t = blockIdx.x ? (int)blockIdx.x - 1 : P.tiles_x * P.tiles_y;
   // a single problem's 16 x 16 tiles all fit on the GPU beside the gradient
   // kernel's blocks: those without windows wait like the others (290.4 us per
   // sweep at n = 512, m = 128; 292.8 if they leave at once)
-  apply_body<TW, TH, 256, false, (TW * TH > 256)>(P, blockIdx.x % P.tiles_x, blockIdx.x / P.tiles_x);
+  apply_body<TW, TH, 256, false, (TW * TH > 256)>(P, t % P.tiles_x, t / P.tiles_x);
 }
 
 // The precision form's update: the same ordered sum, each window's
@@ -89,7 +94,8 @@ __global__ void __launch_bounds__(256) apply_kernel(ApplyArgs P) {
 __global__ void __launch_bounds__(256) apply_tail_kernel(ApplyArgs P) {
   grid_dep_wait();
   clear_handoff(P);
-  apply_body<16, 16, 256, true>(P, blockIdx.x % P.tiles_x, blockIdx.x / P.tiles_x);
+  const int t = blockIdx.x ? (int)blockIdx.x - 1 : P.tiles_x * P.tiles_y;  // the partial sums first, as above
+  apply_body<16, 16, 256, true>(P, t % P.tiles_x, t / P.tiles_x);
 }
 
 // Several problems in one launch (1-D grid): problem i owns blocks
