@@ -1498,10 +1498,12 @@ int enqueue_precision_g0(magpie_ctx* c, const int32_t* idx, int count, cudaStrea
 }
 
 // ev (optional): four events recorded before/after the window kernel and
-// before/after the apply kernel.  own_idx: idx lies in the context's own
-// permutation, final before the stream's previous kernel began.
+// before/after the apply kernel.  sweep: a step of a sweep, which takes the
+// sweep's kernels.  final_idx: idx was final before the stream's previous
+// kernel began, so that it may be read before the wait for that kernel (every
+// step of a sweep but one whose predecessor is the copy of the permutation).
 int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, const cudaEvent_t* ev = nullptr,
-                 bool own_idx = false) {
+                 bool sweep = false, bool final_idx = false) {
   NvtxRange range("magpie minibatch step");
   StepArgs a = make_args(c, idx);
   // the float-atomic update serves the FP32 window phase without the phase
@@ -1515,7 +1517,7 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
   // they run (us per step, early / not: m = 32, n = 400: B = 8 6.7 / 7.4, 32 7.7 /
   // 8.7, 64 8.9 / 9.2, 128 9.8 / 9.2; m = 16: B = 16 6.2 / 6.7, 256 7.7 / 8.2),
   // which also serves deterministic = 0 better than the atomics (B = 32: 9.2)
-  const bool early = own_idx && c->p.m <= 32 && (long long)c->p.minibatch * c->M <= 65536 && !a.phase && !c->cnn &&
+  const bool early = sweep && c->p.m <= 32 && (long long)c->p.minibatch * c->M <= 65536 && !a.phase && !c->cnn &&
                      !c->p.update_probe && !c->precision && !c->stamps;
   const bool atom = c->acc && !early && !c->precision && !c->cnn && !a.phase &&
                     (!split || (c->p.m == 64 && c->p.minibatch >= 64));
@@ -1536,7 +1538,7 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
     a.grad_only = c->cnn ? 1 : 0;
     if (split) {
       if (atom) a.acc = c->acc;
-      CUDA_TRY(split_launch_m(c->p.m, atom, own_idx, a, count, st));
+      CUDA_TRY(split_launch_m(c->p.m, atom, final_idx, a, count, st));
     } else if (a.phase) {
       CUDA_TRY(launch_window_m<kStepRecycle>(c->p.m, a, count, st));
     } else if (atom) {
@@ -1646,7 +1648,7 @@ int capture_sweep(magpie_ctx* c, cudaGraphExec_t* out) {
   CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   int rc = MAGPIE_OK;
   for (int s = 0; s < N && rc == MAGPIE_OK; s += B)
-    rc = enqueue_step(c, c->order + s, N - s < B ? N - s : B, c->cap_stream, nullptr, true);
+    rc = enqueue_step(c, c->order + s, N - s < B ? N - s : B, c->cap_stream, nullptr, true, true);
   cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
   if (rc) {
     if (g) cudaGraphDestroy(g);
@@ -1668,7 +1670,7 @@ int launch_sweep(magpie_ctx* c) {
     const int N = c->p.n_pos, B = c->p.minibatch;
     for (int s = 0; s < N; s += B) {
       // the first step's predecessor is the copy of the permutation itself
-      const int rc = enqueue_step(c, c->order + s, std::min(B, N - s), c->stream, nullptr, s > 0);
+      const int rc = enqueue_step(c, c->order + s, std::min(B, N - s), c->stream, nullptr, true, s > 0);
       if (rc) return rc;
     }
     return capture_sweep(c, &c->graph);
@@ -2228,7 +2230,7 @@ int magpie_profile_sweep(magpie_ctx* c, const int32_t* order, double* window_ms,
   }
   const int N = c->p.n_pos, B = c->p.minibatch;
   for (int s = 0, i = 0; s < N; s += B, ++i) {
-    int rc = enqueue_step(c, c->order + s, N - s < B ? N - s : B, c->stream, &c->events[4 * (size_t)i]);
+    int rc = enqueue_step(c, c->order + s, N - s < B ? N - s : B, c->stream, &c->events[4 * (size_t)i], true, s > 0);
     if (rc) return rc;
   }
   CUDA_TRY(cudaStreamSynchronize(c->stream));
