@@ -93,9 +93,11 @@ typedef struct {
  *      accumulators (16 n_rows n_cols bytes) with 16-byte float atomics, and a
  *      streaming kernel applies N / D and clears them: faster, but the
  *      order of the floating-point sums varies from run to run.
- * With deterministic = 0 the library may take the ordered update where that is
- * the faster of the two (windows of 128 and more, and small minibatches).  The
- * atomic update serves the FP32 window kernel (with or without the probe step); the precision form, the learned correction, the phase rule of
+ * With deterministic = 0 the library takes the ordered update where that is the
+ * faster of the two: windows of 128 and more with at most five levels and
+ * without the probe step, minibatches of fewer than 64 windows of 64 with at
+ * most four, sweeps whose minibatches hold at most 65536 pixels of windows of
+ * 32 and less.  The precision form, the learned correction, the phase rule of
  * Eq. (specification) and context groups always use the ordered update.
  */
 
@@ -124,9 +126,9 @@ typedef struct {
  *                 context stores the amplitudes sqrt(d_k) in its own buffer.
  *   stream      : cudaStream_t (as void*) on which every call is ordered.
  * The context owns its workspaces: amplitudes (4 N m^2 bytes), the per-level
- * probe factors, the minibatch increment buffer (8 B m^2 bytes), with
- * deterministic = 0 the object-sized accumulators (16 n_rows n_cols bytes),
- * and small per-window arrays.  Returns MAGPIE_EINVAL for bad sizes, NULL
+ * probe factors, the minibatch increment buffer (8 B m^2 bytes), where its
+ * steps use the float atomics the object-sized accumulators (16 n_rows n_cols
+ * bytes), and small per-window arrays.  Returns MAGPIE_EINVAL for bad sizes, NULL
  * pointers, out-of-range positions or a deterministic value other than 0 or
  * 1, MAGPIE_EUNSUPPORTED for an m without a kernel.
  */

@@ -888,6 +888,15 @@ int step_slots(const magpie_ctx* c) {
   return c->precision ? c->p.m / kTcLines : split_form(c) ? c->p.m / Split<256>::NL : cluster_of(c->p.m);
 }
 
+// Whether the plain FP32 steps of a deterministic = 0 context (without the
+// phase rule or the learned correction) use the float atomics, for `split`
+// (split_form) or the cluster kernel.  The split form takes the ordered update
+// where that is the faster of the two, as its gradient kernel waits for the
+// atomics (m = 128, B = 64: 23.6 us per step against 21.0; m = 256, B = 64:
+// 70.9 against 63.7; m = 64, B = 16: 10.3 against 9.8, B = 64: 11.8 against
+// 11.9, B = 256: 20.5 against 21.7).
+bool atomic_form(const magpie_ctx* c, bool split) { return !split || (c->p.m == 64 && c->p.minibatch >= 64); }
+
 // ------------------------------------------------- learned coarse correction
 int cnn_side_in(int h, int l) {
   int s = h;
@@ -1506,12 +1515,6 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
                  bool sweep = false, bool final_idx = false) {
   NvtxRange range("magpie minibatch step");
   StepArgs a = make_args(c, idx);
-  // the float-atomic update serves the FP32 window phase without the phase
-  // rule or the learned correction; every other form uses the ordered one, and
-  // so does the split form where that is the faster of the two: its gradient
-  // kernel waits for the atomics (m = 128, B = 64: 23.6 us per step against
-  // 21.0; m = 256, B = 64: 70.9 against 63.7; m = 64, B = 16: 10.3 against
-  // 9.8, B = 64: 11.8 against 11.9, B = 256: 20.5 against 21.7)
   const bool split = split_form(c);
   // a sweep's small windows, up to 64 of 32 x 32: the update lists them while
   // they run (us per step, early / not: m = 32, n = 400: B = 8 6.7 / 7.4, 32 7.7 /
@@ -1519,8 +1522,9 @@ int enqueue_step(magpie_ctx* c, const int32_t* idx, int count, cudaStream_t st, 
   // which also serves deterministic = 0 better than the atomics (B = 32: 9.2)
   const bool early = sweep && c->p.m <= 32 && (long long)c->p.minibatch * c->M <= 65536 && !a.phase && !c->cnn &&
                      !c->p.update_probe && !c->precision && !c->stamps;
-  const bool atom = c->acc && !early && !c->precision && !c->cnn && !a.phase &&
-                    (!split || (c->p.m == 64 && c->p.minibatch >= 64));
+  // the float-atomic update serves the FP32 window phase without the phase
+  // rule or the learned correction; every other form uses the ordered one
+  const bool atom = c->acc && !early && !c->precision && !c->cnn && !a.phase && atomic_form(c, split);
   if (ev) CUDA_TRY(cudaEventRecord(ev[0], st));
   int rc = MAGPIE_OK;
   if (c->precision) {
@@ -2163,7 +2167,8 @@ int magpie_create(magpie_ctx** out, const magpie_params* params, void* object, c
       (rc = alloc((void**)&c->iota, sizeof(int32_t) * N)) || (rc = alloc((void**)&c->order, sizeof(int32_t) * N)) ||
       (rc = alloc((void**)&c->sums, sizeof(double) * 2)) || (rc = alloc((void**)&c->err, sizeof(int))) ||
       (p.levels >= 2 && (rc = alloc((void**)&c->wz, sizeof(float) * M * 2))) ||
-      (!p.deterministic && (rc = alloc((void**)&c->acc, sizeof(float4) * (size_t)p.n_rows * p.n_cols))))
+      (!p.deterministic && atomic_form(c, split_form(c)) &&
+       (rc = alloc((void**)&c->acc, sizeof(float4) * (size_t)p.n_rows * p.n_cols))))
     return rc;
 
   auto cleanup_fail = [&](int code) {
@@ -3194,6 +3199,11 @@ int magpie_stage_times(magpie_ctx* c, const int32_t* idx, int32_t count, uint64_
   if (c->precision || c->cnn) return fail(MAGPIE_EINVAL, "per-stage timestamps time the FP32 window kernel");
   const size_t n = (size_t)count * cluster_of(c->p.m) * kStages;
   if (capacity < (int64_t)n) return fail(MAGPIE_EINVAL, "capacity below count * blocks per window * stages");
+  if (!c->p.deterministic && !c->acc) {  // the stamped cluster kernel uses the atomics where the split form does not
+    const size_t bytes = sizeof(float4) * (size_t)c->p.n_rows * c->p.n_cols;
+    CUDA_TRY(cudaMalloc((void**)&c->acc, bytes));
+    CUDA_TRY(cudaMemsetAsync(c->acc, 0, bytes, c->stream));
+  }
   CUDA_TRY(cudaMalloc(&c->stamps, sizeof(unsigned long long) * n));
   cudaError_t e = cudaMemsetAsync(c->stamps, 0, sizeof(unsigned long long) * n, c->stream);
   int rc = e == cudaSuccess ? enqueue_step(c, idx, count, c->stream) : MAGPIE_OK;

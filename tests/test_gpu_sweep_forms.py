@@ -56,3 +56,36 @@ def test_every_sweep_takes_the_sweeps_kernels(spec):
         assert torch.equal(z_ordered, z_fast), (i, call)
     ordered.close()
     fast.close()
+
+
+# (m, levels, minibatch, update_probe): whether steps of deterministic = 0 use the float atomics
+MEMORY = [(128, 3, 8, 0, False), (256, 5, 2, 0, False), (64, 3, 8, 0, False), (64, 3, 64, 0, True), (64, 3, 128, 0, True),
+          (64, 5, 8, 0, True), (128, 3, 8, 1, True), (128, 6, 8, 0, True), (32, 2, 8, 0, True)]
+
+
+@pytest.mark.parametrize("m,levels,minibatch,probe,atomic", MEMORY)
+def test_accumulators_are_held_where_steps_use_them(m, levels, minibatch, probe, atomic):
+    """Device memory that deterministic = 0 adds to a context on 3000 x 3000
+    pixels: 16 bytes per pixel (137 MiB) or nothing, to allocation granularity."""
+    n, N = 3000, 128
+    dev = torch.device("cuda")
+    z = torch.ones((n, n), dtype=torch.complex64, device=dev)
+    Q = torch.from_numpy(synth.make_probe(m).astype(np.complex64)).to(dev)
+    pos = torch.from_numpy(np.random.default_rng(m).integers(0, n - m + 1, (N, 2)).astype(np.int32)).to(dev)
+    d = magpie.magpie_forward_intensities(z, Q, pos, m)
+
+    def used(deterministic):
+        p = magpie.magpie_params_of(n, n, m, N, levels, minibatch, 0.1, probe, 0.1, deterministic)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx = magpie.magpie_create(p, z, Q, pos, d)
+        taken = before - torch.cuda.mem_get_info()[0]
+        magpie.magpie_step(ctx, torch.arange(8 if minibatch > 8 else minibatch, dtype=torch.int32, device=dev))
+        magpie.magpie_sync(ctx)
+        ctx.close()
+        return taken
+
+    used(1)  # whatever the first context of a side leaves behind
+    extra = used(0) - used(1)
+    granule = 2 << 20
+    assert abs(extra - (16 * n * n if atomic else 0)) <= 4 * granule, extra
