@@ -220,11 +220,12 @@ cudaError_t window_sim_launch(const StepArgs& a, const float2* tw, int windows, 
 template <int MS>
 cudaError_t split_launch(bool atomic, bool early, const StepArgs& a, int windows, cudaStream_t st) {
   using S = Split<MS>;
+  if (atomic && MS != 64) return cudaErrorInvalidValue;  // atomic_form: no other side uses the float atomics
   const dim3 grid((unsigned)windows * S::TILES), block(S::T);
   cudaError_t e = launch_ex(split_exit_kernel<MS>, grid, block, 0, st, 1, true, a, early);
   if (e == cudaSuccess) e = launch_ex(split_project_kernel<MS>, grid, block, 0, st, 1, true, a);
   if (e == cudaSuccess)
-    e = launch_ex(atomic ? split_grad_kernel<MS, true> : split_grad_kernel<MS, false>, grid, block, 0, st, 1, true, a);
+    e = launch_ex(atomic ? split_grad_kernel<MS, MS == 64> : split_grad_kernel<MS, false>, grid, block, 0, st, 1, true, a);
   return e;
 }
 
