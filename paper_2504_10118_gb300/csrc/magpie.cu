@@ -1669,6 +1669,9 @@ int capture_sweep(magpie_ctx* c, cudaGraphExec_t* out) {
 // first sweep of a context is launched step by step, and its graph is captured
 // while the GPU runs it (first sweep of the n = 512, m = 128, 900-window
 // problem, which waited for capture and instantiation before: 441 -> 332 us).
+// A capture that fails then (out of memory, say) is no error of this sweep,
+// which is in the stream and will change the object: the next sweep is
+// launched step by step as well, and captured again.
 int launch_sweep(magpie_ctx* c) {
   if (!c->graph) {
     const int N = c->p.n_pos, B = c->p.minibatch;
@@ -1677,7 +1680,11 @@ int launch_sweep(magpie_ctx* c) {
       const int rc = enqueue_step(c, c->order + s, std::min(B, N - s), c->stream, nullptr, true, s > 0);
       if (rc) return rc;
     }
-    return capture_sweep(c, &c->graph);
+    if (capture_sweep(c, &c->graph)) {
+      c->graph = nullptr;
+      cudaGetLastError();
+    }
+    return MAGPIE_OK;
   }
   CUDA_TRY(cudaGraphLaunch(c->graph, c->stream));
   return MAGPIE_OK;
