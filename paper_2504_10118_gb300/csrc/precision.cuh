@@ -871,8 +871,10 @@ __global__ void __launch_bounds__(1024) coarse_cycle_kernel(const PrecArgs A) {
   constexpr int nt = 1024;
   const int w = blockIdx.x, q = blockIdx.y, tid = threadIdx.x, L = A.L;
   grid_dep_launch();  // the update kernel after it waits for the whole grid
-  if ((unsigned)A.idx[w] >= (unsigned)A.n_pos) return;
+  // (skipped windows as well: their gradient blocks count their tiles too, and
+  // the update clears the counts once this grid has ended)
   if (!handoff_wait(A, &A.hand[2 * A.count + w], MS / kTcLines)) return;  // ran out: skip the window
+  if ((unsigned)A.idx[w] >= (unsigned)A.n_pos) return;
   auto off = [&](int l) {  // level l >= 2
     int o = 0;
     for (int j = 2; j < l; ++j) o += (MS >> j) * (MS >> j);

@@ -103,3 +103,28 @@ def test_group_sweep_of_skipped_windows_changes_nothing():
     group.close()
     for c in ctxs:
         c.close()
+
+
+@pytest.mark.parametrize("path", [1, 2])
+@pytest.mark.parametrize("m,levels", [(64, 3), (64, 6), (128, 7)])
+def test_precision_steps_with_skipped_windows(m, levels, path):
+    """Tensor-core steps hand windows from kernel to kernel by counts that the
+    update clears: skipped windows, some or all of a step's, leave the counts and
+    the object as a step without them does (the V-cycle inside the gradient
+    kernel, and the coarse kernel of deeper cycles)."""
+    mb = member(m, levels)
+    ctx = mb.ctx()
+    z = mb.zt
+    plain = mb.ctx()
+    z_plain = mb.zt
+    for c in (ctx, plain):
+        magpie.magpie_set_precision(c, path)
+    for r in range(ROUNDS):
+        k = r % mb.N
+        magpie.magpie_step(ctx, dev_idx([mb.N, k, -1, (k + 2) % mb.N]))
+        magpie.magpie_step(ctx, dev_idx([mb.N + r] if r % 2 else [-1, mb.N, mb.N + 3]))
+        magpie.magpie_step(plain, dev_idx([k, (k + 2) % mb.N]))
+        assert torch.equal(z, z_plain)
+        reported(ctx)
+    ctx.close()
+    plain.close()
