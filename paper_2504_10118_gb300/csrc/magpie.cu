@@ -1671,9 +1671,14 @@ int capture_sweep(magpie_ctx* c, cudaGraphExec_t* out) {
 // problem, which waited for capture and instantiation before: 441 -> 332 us).
 // A capture that fails then (out of memory, say) is no error of this sweep,
 // which is in the stream and will change the object: the next sweep is
-// launched step by step as well, and captured again.
+// launched step by step as well, and captured again.  On a stream that is
+// itself being captured no sweep runs, a first one no more than a replay.
 int launch_sweep(magpie_ctx* c) {
   if (!c->graph) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(c->stream, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone)
+      return fail(MAGPIE_ECUDA, "a sweep cannot be captured: its steps replay a graph of their own");
     const int N = c->p.n_pos, B = c->p.minibatch;
     for (int s = 0; s < N; s += B) {
       // the first step's predecessor is the copy of the permutation itself
@@ -1686,7 +1691,9 @@ int launch_sweep(magpie_ctx* c) {
     }
     return MAGPIE_OK;
   }
-  CUDA_TRY(cudaGraphLaunch(c->graph, c->stream));
+  const cudaError_t e = cudaGraphLaunch(c->graph, c->stream);
+  if (e != cudaSuccess) cudaGetLastError();  // this call's error, not that of the next launch that is checked
+  CUDA_TRY(e);
   return MAGPIE_OK;
 }
 

@@ -76,3 +76,44 @@ def test_failed_capture_is_no_error_of_the_sweep_that_ran(faked, spec):
     magpie.magpie_sync(ctx)
     ctx.close()
     plain.close()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_no_sweep_on_a_stream_that_is_captured(warm):
+    """Refused with an error, the object untouched, the context usable after."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    magpie.build()
+    mb = Member((75, 32, 5, 9, 1, 2, 8), 6)
+    plain = mb.ctx()
+    z_plain = mb.zt
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        ctx = mb.ctx()
+        z = mb.zt
+        o = orders([mb], 0)[0]
+        if warm:
+            magpie.magpie_sweep(ctx, o)
+        stream.synchronize()
+        before = z.clone()
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin()
+        with pytest.raises(magpie.MagpieError) as ei:
+            magpie.magpie_sweep(ctx, o)
+        try:
+            graph.capture_end()
+        except RuntimeError:
+            pass  # the refused call may have invalidated the capture
+        assert ei.value.code == magpie.ECUDA
+        stream.synchronize()
+        assert torch.equal(z, before)
+        magpie.magpie_sweep(ctx, o)
+        stream.synchronize()
+    for _ in range(1 + warm):
+        magpie.magpie_sweep(plain, o)
+    torch.cuda.synchronize()
+    assert torch.equal(z, z_plain)
+    ctx.close()
+    plain.close()
