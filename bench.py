@@ -547,7 +547,7 @@ def sweeps_to_nrmse(w, dev, magpie, target: float, max_sweeps: int, every: int =
     wall = time.perf_counter() - t0
     out = {"levels": w.levels, "minibatch": w.minibatch, "alpha": w.alpha, "reached": err <= target,
            "sweeps": sweeps, "seconds": ms * 1e-3, "wall_seconds": wall, "nrmse": err, "best_nrmse": best,
-           "update": "ordered" if deterministic else "atomic",
+           "update": "ordered" if precision or net is not None else update_of(w, deterministic),
            "dft": {1: "tensor-core FP16 hi+lo (mma.sync)", 2: "tensor-core FP16 hi+lo (tcgen05)"}.get(precision,
                                                                                               "FP32 FFT"),
            "learned": net is not None}
@@ -729,6 +729,16 @@ def split_form(w) -> bool:
     return w.m >= 64 and w.levels <= (5 if w.m >= 128 else 4) and not (w.m == 64 and 64 < w.minibatch <= 152)
 
 
+def update_of(w, deterministic: int) -> str:
+    """The update that a sweep of the FP32 form of this workload takes.  With
+    deterministic = 0 the library takes the ordered one where that is faster:
+    the strip kernels' steps but those of 64 and more windows of 64, and sweeps
+    whose minibatches hold at most 65536 pixels of windows of 32 and less."""
+    if deterministic or (w.m <= 32 and w.minibatch * w.m * w.m <= 65536):
+        return "ordered"
+    return "ordered" if split_form(w) and not (w.m == 64 and w.minibatch >= 64) else "atomic"
+
+
 def step_launches(args, w) -> int:
     """launches_per_step with the library's forms for this workload: windows of
     64 and more run their window phase as three kernels, the precision form's
@@ -837,11 +847,15 @@ def run_ours(args, w):
     alu_peak, alu_src = fp32_peak(dev, magpie)
     achieved_tf = windows * flops_per_window(w.m) / (wk_ms * 1e-3) / 1e12
     achieved_gbs = windows * hbm_bytes_per_window(w.m) / (wk_ms * 1e-3) / 1e9
-    traffic = measured_traffic(det, split_form(w)) if fp32_form else None
+    traffic = measured_traffic(1 if update_of(w, det) == "ordered" else 0, split_form(w)) if fp32_form else None
 
     # the other update of the FP32 form on the same data, timed the same way
+    # (where deterministic = 0 takes the ordered update there is no other)
     update_ab = None
-    if fp32_form and rank == 0 and world == 1:
+    if fp32_form and rank == 0 and world == 1 and update_of(w, 0) == "ordered":
+        update_ab = {"headline": "ordered", "note": "sweeps of this workload take the ordered update for both values of "
+                                                    "deterministic: one set of kernels, timed once"}
+    elif fp32_form and rank == 0 and world == 1:
         z2 = torch.ones((w.n, w.n), dtype=torch.complex64, device=dev)
         ctx2 = magpie.magpie_create(magpie.magpie_params_of(w.n, w.n, w.m, w.n_pos, w.levels, w.minibatch, w.alpha,
                                                             deterministic=1 - det), z2, Qt, post, dt)
@@ -861,8 +875,7 @@ def run_ours(args, w):
                                                      "window_kernel_ms_per_sweep": wk2 / prof_sweeps,
                                                      "update_kernel_ms_per_sweep": ap2 / prof_sweeps}}
         update_ab = dict(rec, headline=args.update,
-                         note="same data and sweep orders; per-kernel times from event-bracketed launches; windows "
-                              "of 128 and more take the ordered update for both values of the parameter")
+                         note="same data and sweep orders; per-kernel times from event-bracketed launches")
 
     # end to end through the host-buffer call: order + intensities in, object out
     order_h = [torch.from_numpy(synth.make_order(w.n_pos, 1000 + s)).pin_memory() for s in range(max(2, args.steps))]
@@ -912,7 +925,7 @@ def run_ours(args, w):
                            dft={"tc": "tensor-core FP16 hi+lo (mma.sync)",
                                 "tcgen05": "tensor-core FP16 hi+lo (tcgen05, TMEM accumulators)"}.get(args.dft,
                                                                                                   "FP32 FFT"),
-                           update="ordered" if det else "atomic"),
+                           update=update_of(w, det) if fp32_form else "ordered", deterministic=det),
             "quality": quality,
             "update_ab": update_ab,
             "time_to_nrmse": ttn,
@@ -923,7 +936,7 @@ def run_ours(args, w):
             "roofline": ({"bound": "alu", "achieved": achieved_tf, "peak": alu_peak, "unit": "TFLOP/s",
                          "frac": achieved_tf / alu_peak, "traffic": traffic,
                          "kernel": (f"split_exit/project/grad_kernel<{w.m}> (one window phase)" if split_form(w)
-                                    else f"window_kernel<{w.m}, {'step' if det else 'step_atomic'}>"),
+                                    else f"window_kernel<{w.m}, {'step' if update_of(w, det) == 'ordered' else 'step_atomic'}>"),
                          "avg_launch_ms": wk_ms / max(launches, 1),
                          "flops_per_window": flops_per_window(w.m),
                          "peak_source": alu_src,
@@ -962,8 +975,9 @@ def main():
                     help="fft: FP32 FFT path; tc: tensor-core FP16 hi+lo DFTs on mma.sync (default for the "
                          "precision workload); tcgen05: the same DFTs on tcgen05 with TMEM accumulators")
     ap.add_argument("--update", choices=["atomic", "ordered"], default="atomic",
-                    help="update of the FP32 form: float-atomic accumulation (default) or the ordered, bitwise "
-                         "reproducible reduction; the other one is timed too (update_ab)")
+                    help="update of the FP32 form: deterministic = 0 (default; float-atomic accumulation, or the "
+                         "ordered update where that is faster) or the ordered, bitwise reproducible reduction; where "
+                         "the two differ the other one is timed too (update_ab)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-extras", action="store_true",
                     help="skip the time-to-NRMSE, precision and batched records of the default workload")
