@@ -18,10 +18,10 @@ namespace magpie_impl {
 
 namespace cg = cooperative_groups;
 
-constexpr int kMaxMinibatch = 4096;  // the update kernel keeps the minibatch's corners in smem (48 KiB)
+constexpr int kMaxMinibatch = 4096;  // the update kernel lists the minibatch's windows in smem (16 bytes each: 64 KiB)
 constexpr int kMaxCluster = 8;       // largest number of blocks per window
-constexpr int kMaxSlots = 16;        // partial-sum slots per window: the window kernel's blocks, or m / 16
-                                     // blocks of the precision form (m <= 256)
+constexpr int kMaxSlots = 16;        // partial-sum slots per window: the window kernel's blocks, or the
+                                     // m / 16 blocks of the split and the precision form (m <= 256)
 constexpr int kApplyUnroll = 4;      // increments in flight per thread in the update kernel
 
 #include "fft_lines.cuh"

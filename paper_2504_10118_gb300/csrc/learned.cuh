@@ -1,7 +1,7 @@
 // learned.cuh -- the learned coarse-level correction: the network's forward
-// pass (BF16 tensor-core implicit GEMM, FP32 accumulation), its backward pass
-// and Adam step (FP32), and the per-window kernels that build the network's
-// input on the coarsest grid of the V-cycle and apply its proposal with the
+// pass (BF16 tensor-core implicit GEMM, FP32 accumulation), its Adam step
+// (FP32; the backward pass is in learned_backward.cuh), and the per-window
+// kernels that build the network's input on the coarsest grid of the V-cycle and apply its proposal with the
 // surrogate acceptance test.  Included by magpie.cu inside its anonymous
 // namespace.
 //

@@ -61,7 +61,7 @@ constexpr int kVersion = 10300;  // 1.3.0
 #include "precision.cuh"
 
 // The precision form's window hand-off counts are final once the update
-// kernel that ends the step may run: block (0, 0) zeroes them for the next
+// kernel that ends the step may run: block 0 zeroes them for the next
 // step (whose exit kernel waits for this grid to complete).
 __device__ __forceinline__ void clear_handoff(const ApplyArgs& P) {
   if (P.hand && blockIdx.x == 0)
@@ -871,7 +871,11 @@ StepArgs make_args(magpie_ctx* c, const int32_t* idx) {
 // so do m = 64 minibatches beyond 64 windows that still run at once on two
 // blocks per SM (152 clusters of two).  us per step, three levels, ordered
 // update (split / cluster kernel):
-//   m = 64, n = 300   B = 16: 9.8 / 10.8, 64: 11.9 / 12.2, 128: 15.4 / 14.4, 512: 35.7 / 47.3
+//   m = 64, n = 300   B = 16: 9.8 / 10.8, 64: 11.9 / 12.2, 512: 35.7 / 47.3
+//     sweeps, n = 300  B = 80: 12.6 / 13.0, 96: 13.8 / 13.3, 128: 15.5 / 14.0, 152: 16.5 / 14.4
+//             n = 600  B = 80: 12.4 / 13.7, 96: 12.8 / 14.0, 128: 14.6 / 14.4, 152: 15.3 / 14.9
+//             n = 1024 B = 80: 13.1 / 14.5, 96: 13.9 / 14.8, 128: 15.9 / 15.4, 152: 17.0 / 15.9
+//     (so the line holds from 120 windows on, and from 90 where they overlap densely)
 //   m = 128, n = 512  B = 4: 11.3 / 14.9, 16: 14.9 / 16.7, 64: 20.7 / 22.0, 256: 57.8 / 66.7
 //   m = 256, n = 800  B = 4: 16.6 / 27.3, 16: 27.1 / 50.0, 64: 57.9 / 117
 // A function of the context alone, so that a member of a group takes the same
@@ -893,8 +897,12 @@ int step_slots(const magpie_ctx* c) {
 // (split_form) or the cluster kernel.  The split form takes the ordered update
 // where that is the faster of the two, as its gradient kernel waits for the
 // atomics (m = 128, B = 64: 23.6 us per step against 21.0; m = 256, B = 64:
-// 70.9 against 63.7; m = 64, B = 16: 10.3 against 9.8, B = 64: 11.8 against
-// 11.9, B = 256: 20.5 against 21.7).
+// 70.9 against 63.7; m = 64, B = 16: 10.3 against 9.8).  With 64 and more
+// windows of 64 the atomics are the faster ones where the windows overlap
+// densely (sweeps, us per step, atomic / ordered: n = 200 B = 64 11.3 / 12.3,
+// 256 20.4 / 25.0, 512 32.1 / 41.6; n = 300 11.3 / 11.5, 20.2 / 20.2, 32.1 / 31.7)
+// and the slower ones on larger objects (n = 600 12.0 / 11.4, 20.9 / 19.3, 32.8 /
+// 30.4; n = 1024 13.1 / 12.0, 21.8 / 21.1, 34.4 / 32.1).
 bool atomic_form(const magpie_ctx* c, bool split) { return !split || (c->p.m == 64 && c->p.minibatch >= 64); }
 
 // ------------------------------------------------- learned coarse correction
@@ -1239,7 +1247,9 @@ CoarseArgs coarse_args(magpie_ctx* c, const int32_t* idx, float4* x, float* scal
 
 cudaError_t launch_coarse_state(const CoarseArgs& a, int count, cudaStream_t st) {
   // the cluster kernels store whole float4 (a caller's x may be less aligned) and
-  // keep at most four coarse pixels per thread
+  // keep at most four coarse pixels per thread, each with its fine pixels' loads
+  // unrolled: two to four levels.  Five (m = 128, h = 8: 256 fine pixels behind
+  // each of 64 coarse ones) keep the one-block kernel and its launch boundary.
   const bool fits = ((uintptr_t)a.x & 15) == 0 && (a.MS >> (a.L - 1)) <= 64;
   const dim3 grid(4 * (unsigned)count), block(256);
   if (fits && a.L == 2) return launch_ex(coarse_state_cluster_kernel<2>, grid, block, 0, st, 4, true, a);

@@ -10,9 +10,9 @@
 // as recorded by the window kernel; a ballot compaction over all warps), each
 // with its increments' offset; each thread then walks that list a few entries
 // at a time with predicated loads, so several increments are in flight per
-// thread.  The block after the last tile turns the window kernel's block
-// partials into Phi_k and ||grad Phi_k||, beside the tiles rather than before
-// one of them.  Dynamic smem: count entries.  Every tile shape sums each
+// thread.  Tile number tiles_x tiles_y turns the window phase's block partials
+// into Phi_k and ||grad Phi_k||, in a block of its own beside the tiles.
+// Dynamic smem: count entries.  Every tile shape sums each
 // pixel's windows in minibatch order, so all give bitwise equal objects.
 struct ApplyShape {
   int tw, th;
@@ -39,7 +39,7 @@ struct ApplyArgs {
   const float2* e1;        // [count][MS/2][MS/2] e^1
   const float* u0;         // [MS][MS] u^0
   int* hand;               // precision form: the step's window hand-off counts, zeroed by
-  int nhand;               // block (0, 0) once the grid may run (null otherwise)
+  int nhand;               // block 0 once the grid may run (null otherwise)
   int early;               // the object and the windows' positions are final before the stream's previous
                            // kernel ends: the windows are listed before the wait for it, their corners
                            // as an earlier kernel recorded them (1) or from idx and pos (2)
@@ -77,7 +77,7 @@ __device__ __forceinline__ void apply_body(const ApplyArgs& P, const int tx, con
   ApplyEntry* list = reinterpret_cast<ApplyEntry*>(apply_smem);
   __shared__ int warp_hits[NW];
   if (!P.early) grid_dep_wait();
-  if (ty >= P.tiles_y) {  // the block after the last tile
+  if (ty >= P.tiles_y) {  // the partial sums' block
     if (P.early) {
       grid_dep_wait();
       grid_dep_launch();

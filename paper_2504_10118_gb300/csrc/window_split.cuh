@@ -21,8 +21,8 @@
 // 15 x 8 of the 152 SMs with one block each at m = 256, and waited twice per
 // window for exchanges through distributed shared memory.  Sweeps (GB300, us,
 // cluster kernel / split form): n = 1024, m = 256, 2500 windows, 4 levels,
-// minibatch 64: 5240 / 2250; n = 512, m = 128, 900 windows, 3 levels,
-// minibatch 64: 321 / 291.  Of the 56 us of an m = 256 step the kernels alone
+// minibatch 64: 5240 / 2210; n = 512, m = 128, 900 windows, 3 levels,
+// minibatch 64: 321 / 290.  Of the 56 us of an m = 256 step the kernels alone
 // take 12.6, 16.5, 19.4 and the update 9 us.  Tried and left out: handing
 // windows from kernel to kernel one by one with counters (2.86 ms against
 // 2.54: the waiting blocks hold the slots of working ones), loading z and Q
