@@ -503,9 +503,11 @@ int apply_tiles(const ApplyArgs& P) { return P.tiles_x * P.tiles_y + 1; }
 // The update of one problem on its own, in the largest of 32 x 32, 32 x 16 and
 // 16 x 16 tiles (four, two and one pixel per thread, which share the window
 // list and its tests) that leaves at least five blocks per SM: smaller grids
-// leave SMs idle.  us per 64-window step, three levels, in that order:
-//   m = 128: n = 512 24.4 / 20.3 / 19.6, 640 23.3 / 21.0 / 21.6, 1024 22.1 / 23.6 / 25.6
-//   m = 256: n = 600 70.9 / 58.3 / 57.7, 1024 56.9 / 56.9 / 59.5 (four levels)
+// leave SMs idle.  us per 64-window step of a sweep, three levels, in that order:
+//   m = 128: n = 300 30.9 / 24.8 / 23.4, 512 21.8 / 19.2 / 18.9, 640 20.2 / 18.6 / 19.0,
+//            760 19.2 / 19.2 / 19.8, 900 18.9 / 20.0 / 21.0, 2048 24.3 / 30.6 / 36.8
+//   m = 256 (four levels): n = 600 61.8 / 55.6 / 55.0, 800 55.0 / 53.7 / 54.1,
+//            1024 54.1 / 54.5 / 55.8, 2048 60.1 / 67.5 / 73.9
 cudaError_t launch_apply_args(ApplyArgs P, cudaStream_t st) {
   struct Tile {
     int w, h;
