@@ -22,7 +22,7 @@
 // window for exchanges through distributed shared memory.  Sweeps (GB300, us,
 // cluster kernel / split form): n = 1024, m = 256, 2500 windows, 4 levels,
 // minibatch 64: 5240 / 2210; n = 512, m = 128, 900 windows, 3 levels,
-// minibatch 64: 321 / 290.  Of the 56 us of an m = 256 step the kernels alone
+// minibatch 64: 321 / 289.  Of the 56 us of an m = 256 step the kernels alone
 // take 12.6, 16.5, 19.4 and the update 9 us.  Tried and left out: handing
 // windows from kernel to kernel one by one with counters (2.86 ms against
 // 2.54: the waiting blocks hold the slots of working ones), loading z and Q
@@ -123,17 +123,15 @@ __device__ __forceinline__ void split_project_body(const StepArgs& A, int win, i
   __shared__ float2 X[NL * MS];
   const int tid = threadIdx.x, rl = tid / G, g = tid % G, kr = tile * NL + rl;
   const int k = A.idx[win];
-  if ((unsigned)k >= (unsigned)A.n_pos) {
-    grid_dep_wait();  // see split_exit_kernel
-    return;
-  }
-  const float* ampr = A.amp + (size_t)k * S::M + kr * MS + g;
+  const bool ok = (unsigned)k < (unsigned)A.n_pos;  // a skipped window waits as well: see split_exit_kernel
+  const float* ampr = A.amp + (size_t)(ok ? k : 0) * S::M + kr * MS + g;
   float av[E];  // fetched while the exit kernel finishes
 #pragma unroll
   for (int j = 0; j < E / G; ++j)
 #pragma unroll
     for (int k2 = 0; k2 < G; ++k2) av[j * G + k2] = __ldg(ampr + G * j + E * k2);
   grid_dep_wait();
+  if (!ok) return;
   grid_dep_launch();
   float2* row = A.contrib + (size_t)win * S::M + kr * MS + g;
   float2 x[E];
@@ -263,15 +261,13 @@ __device__ __forceinline__ void split_grad_body(const StepArgs& A, int win, int 
   __shared__ float2 X[NL * MS];
   const int tid = threadIdx.x, l = tid % NL, g = tid / NL, c = tile * NL + l;
   const int k = A.idx[win];
-  if ((unsigned)k >= (unsigned)A.n_pos) {
-    grid_dep_wait();  // see split_exit_kernel
-    return;
-  }
-  const int pr = A.pos[2 * k], pc = A.pos[2 * k + 1];
+  const bool ok = (unsigned)k < (unsigned)A.n_pos;  // a skipped window waits as well: see split_exit_kernel
+  const int pr = A.pos[ok ? 2 * k : 0], pc = A.pos[ok ? 2 * k + 1 : 1];
   const float2* zp = A.z + (size_t)(pr + g) * A.n_cols + pc + c;
   const float2* qp = A.Q + g * MS + c;
   const size_t zs = (size_t)G * A.n_cols;
   grid_dep_wait();
+  if (!ok) return;
   if (!ATOM) grid_dep_launch();  // the ordered update lists its windows meanwhile
   float2* col = A.contrib + (size_t)win * S::M + c;
   float2 x[E];
