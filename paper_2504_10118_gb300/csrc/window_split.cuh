@@ -322,9 +322,8 @@ __device__ __forceinline__ void split_grad_body(const StepArgs& A, int win, int 
 // where its window is skipped, then lets the next one's blocks be set up, so
 // that a kernel's blocks start once every kernel but the one before theirs has
 // ended: the update reads the corners that the exit kernel wrote before its
-// own wait, which is for the gradient kernel.  (A grid that ended without
-// having waited, as one of skipped windows alone once did, would let the
-// update read the corners of an earlier step.)
+// own wait, which is for the gradient kernel, and would read an earlier step's
+// if a grid of skipped windows ended without having waited.
 template <int MS>
 __global__ void __launch_bounds__(Split<MS>::T, Split<MS>::MB[0]) split_exit_kernel(const __grid_constant__ StepArgs A, bool early) {
   split_exit_body<MS>(A, blockIdx.x / Split<MS>::TILES, blockIdx.x % Split<MS>::TILES, early);
